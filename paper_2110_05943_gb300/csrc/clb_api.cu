@@ -46,6 +46,7 @@ struct clb_handle {
     clb_lattice lat{};
     KParamsT<double> k64{};       // FP64 form
     KParamsT<float> k32{};        // FP16 forms
+    SplitPhys sp{};               // FP64 form: the constants of its split arithmetic
     int prec = CLB_F64;
     size_t es = 8;                // bytes per stored distribution value
     cudaStream_t stream = nullptr;
@@ -59,6 +60,7 @@ struct clb_handle {
     unsigned* seq = nullptr;              // FP16 forms: step counter of each buffer (seeds the rounding)
     int par = 0;
     CoefT<double>* coef = nullptr;   // FP64 form: per-node constants
+    float2* scoef = nullptr;         // and as split numbers, in planes
     float* phi32 = nullptr;          // FP16 forms: porosity (dense) or 1/phi (pitched)
     void* ayg = nullptr;             // a_y - g beta T0 per row (double or float)
     double* scratch = nullptr;       // 4 dense fields (macros, set_fields)
@@ -80,10 +82,10 @@ struct clb_handle {
     unsigned* tma_fail = nullptr;   // device flag set by a CTA whose wait expired
     std::string err;
 
-    AuxT<double> aux64() const { return AuxT<double>{coef, nullptr, nullptr, (const double*)ayg}; }
+    AuxT<double> aux64() const { return AuxT<double>{coef, nullptr, nullptr, (const double*)ayg, scoef}; }
     AuxT<float> aux32() const {
-        return prec == CLB_F16N ? AuxT<float>{nullptr, nullptr, phi32, (const float*)ayg}
-                                : AuxT<float>{nullptr, phi32, nullptr, (const float*)ayg};
+        return prec == CLB_F16N ? AuxT<float>{nullptr, nullptr, phi32, (const float*)ayg, nullptr}
+                                : AuxT<float>{nullptr, phi32, nullptr, (const float*)ayg, nullptr};
     }
     template <typename S>
     BufT<S> buf(int i) const { return BufT<S>{(S*)f[i], (S*)g[i], rec[i], seq ? seq + i : nullptr}; }
@@ -311,6 +313,7 @@ static void free_all(clb_handle* h) {
     }
     cudaFree(h->seq);
     cudaFree(h->coef);
+    cudaFree(h->scoef);
     cudaFree(h->phi32);
     cudaFree(h->ayg);
     cudaFree(h->scratch);
@@ -322,19 +325,19 @@ static void free_all(clb_handle* h) {
 }
 
 // ------------------------------------------------------------------ kernels
-template <class P, typename K>
-static void step_as(clb_handle* h, cudaStream_t s, const AuxT<typename P::R>& A, const K& kp) {
-    using S = typename P::S;
-    const BufT<S> in = h->buf<S>(h->par), out = h->buf<S>(1 - h->par);
+static void step_f64(clb_handle* h, cudaStream_t s) {
+    const BufT<double> in = h->buf<double>(h->par), out = h->buf<double>(1 - h->par);
+    const AuxT<double> A = h->aux64();
+    const KParamsT<double>& K = h->k64;
     const bool sh = h->prm.shift != 0, fo = h->prm.forchheimer != 0;
-    // interior tiles, then the wall nodes (see k_step)
-    const int tx = (int)h->grid.x, nt = (int)(h->grid.x * h->grid.y);
+    // the wall nodes, then interior tiles (see k_step_f64)
     const int threads = (int)(h->block.x * h->block.y);
-    const unsigned nb = (unsigned)(nt + (wall_count(h->k64.g) + threads - 1) / threads);
-    if (sh && fo) k_step<P, true, true><<<nb, h->block, 0, s>>>(in, out, A, kp, tx, nt);
-    else if (sh) k_step<P, true, false><<<nb, h->block, 0, s>>>(in, out, A, kp, tx, nt);
-    else if (fo) k_step<P, false, true><<<nb, h->block, 0, s>>>(in, out, A, kp, tx, nt);
-    else k_step<P, false, false><<<nb, h->block, 0, s>>>(in, out, A, kp, tx, nt);
+    const int tx = (int)h->grid.x, nw = (int)((wall_count(K.g) + threads - 1) / threads);
+    const unsigned nb = (unsigned)nw + h->grid.x * h->grid.y;
+    if (sh && fo) k_step_f64<true, true><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
+    else if (sh) k_step_f64<true, false><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
+    else if (fo) k_step_f64<false, true><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
+    else k_step_f64<false, false><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
 }
 
 // FP16 forms: two nodes per thread (k_step2), grid over node pairs.
@@ -389,7 +392,7 @@ static void step2_as(clb_handle* h, cudaStream_t s, long long limit = TT_LIMIT, 
 static void launch_step(clb_handle* h, cudaStream_t s) {
     if (h->prec == CLB_F16S) step2_as<StoreH16>(h, s);
     else if (h->prec == CLB_F16N) step2_as<StoreH16N>(h, s);
-    else step_as<StoreF64>(h, s, h->aux64(), h->k64);
+    else step_f64(h, s);
     h->par = 1 - h->par;
 }
 
@@ -570,6 +573,9 @@ extern "C" int clb_init(clb_handle** out, const clb_params* p, const double* phi
         for (int i = 1; i < 5; ++i) k.wg[i] = (float)(0.25 * p->varpi * p->T0);
     }
     const Geo& G = h->k64.g;
+    h->sp = split_phys(h->k64.p.sp, h->k64.p.sm, lat.sv, p->s3, p->s4, p->sigma, lat.zeta_a, h->k64.p.cT2,
+                       std::max(std::fabs(p->T0) + p->dT, std::fabs(p->T_init)), h->k64.b.uw, h->k64.b.vw, h->k64.b.Tw,
+                       h->k64.b.iso);
     pick_launch(h);
 
     const size_t fbytes = (size_t)G.plane * 9 * h->es;
@@ -595,7 +601,10 @@ extern "C" int clb_init(clb_handle** out, const clb_params* p, const double* phi
     else if (h->prec == CLB_F16N) {
         CKI(cudaMalloc(&h->phi32, (size_t)G.plane * sizeof(float)));
         CKI(cudaMemsetAsync(h->phi32, 0, (size_t)G.plane * sizeof(float), h->stream));
-    } else CKI(cudaMalloc(&h->coef, (size_t)n * sizeof(CoefT<double>)));
+    } else {
+        CKI(cudaMalloc(&h->coef, (size_t)n * sizeof(CoefT<double>)));
+        CKI(cudaMalloc(&h->scoef, (size_t)n * sizeof(float2) * kSplitPlanes));
+    }
     CKI(cudaMalloc(&h->ayg, (size_t)p->ny * (half ? sizeof(float) : sizeof(double))));
     CKI(cudaMalloc(&h->scratch, (size_t)n * 4 * sizeof(double)));
     CKI(cudaMalloc(&h->snap, (size_t)n * 3 * sizeof(double)));
@@ -618,10 +627,12 @@ extern "C" int clb_init(clb_handle** out, const clb_params* p, const double* phi
     if (half)
         k_phi32<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->scratch, h->phi32, p->nx, p->ny, px,
                                                                       h->prec == CLB_F16N);
-    else
+    else {
         k_coef<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->scratch, (const double*)h->ayg, h->coef,
                                                                      p->nx, n, lat.nu, lat.K, p->ax, lat.gbeta,
                                                                      p->forchheimer);
+        k_split_coef<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->coef, h->scoef, n);
+    }
     CKI(cudaGetLastError());
     CKI(cudaStreamSynchronize(h->stream));
 

@@ -379,6 +379,7 @@ extern "C" int clb_batch_init(clb_batch** out, int32_t ncase, const clb_params* 
             clb_handle* h = b->cases[c];
             t[c].K = h->k64;
             t[c].A = h->aux64();
+            t[c].P = h->sp;
             t[c].b[0] = h->buf<double>(0);
             t[c].b[1] = h->buf<double>(1);
             t[c].flip = 0;

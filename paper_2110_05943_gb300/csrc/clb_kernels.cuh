@@ -45,6 +45,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "clb_split.cuh"
+
 #ifndef CLB_HD
 #define CLB_HD __device__ __forceinline__
 #endif
@@ -114,6 +116,7 @@ struct AuxT {
     const float* phi;
     const float* ip;
     const R* ayg;
+    const float2* scoef;   // FP64 form: the constants as split numbers, kSplitPlanes dense planes
 };
 
 // One ping-pong buffer: distribution planes, and for the equilibrium-shifted
@@ -1329,46 +1332,129 @@ __device__ __forceinline__ void wall_node(const Geo& G, int i, int& x, int& y) {
     y = i < G.ny ? i : i - G.ny;
 }
 
+// ---------------------------------------------------------------- FP64 step
+// The FP64 form's step in split arithmetic (clb_split.cuh): the same nodes,
+// buffers and loads as step_interior / step_wall, the arithmetic on the FP32
+// and integer pipes.  False: the node left the fixed-point range and has not
+// been stored; the caller takes the FP64 path for it.
+__device__ __forceinline__ SplitCoef split_coef(const AuxT<double>& A, const Geo& G, int x, int y) {
+    const long long n = (long long)G.nx * G.ny;
+    const float2* p = A.scoef + ((long long)y * G.nx + x);
+    sf v[kSplitPlanes];
+#pragma unroll
+    for (int k = 0; k < kSplitPlanes; ++k) {
+        const float2 t = __ldg(p + k * n);
+        v[k] = sf{t.x, t.y};
+    }
+    return SplitCoef{v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]};
+}
+
+template <class L>
+__device__ __forceinline__ void split_pull(const BufT<double>& in, const Geo& G, const SplitPhys& P, int x, int y,
+                                           long long (&f)[9], long long (&g)[5], uint32_t& range, uint32_t& big) {
+    long long o[9];
+    sources<long long>(G, x, y, o);
+    double vf[9], vg[5];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) vf[i] = L::ld(in.f + i * G.plane + o[i]);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) vg[i] = L::ld(in.g + i * G.plane + o[i]);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = fix_f(vf[i], range);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) g[i] = fix_g(vg[i], P.gexp, big);
+}
+
+__device__ __forceinline__ void split_store(const BufT<double>& out, const Geo& G, const SplitPhys& P, int x, int y,
+                                            const long long (&f)[9], const long long (&g)[5]) {
+    const long long o = (long long)y * G.px + x;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) __stwb(out.f + i * G.plane + o, unfix(f[i]));
+#pragma unroll
+    for (int i = 0; i < 5; ++i) __stwb(out.g + i * G.plane + o, unfix(g[i], 60 - P.gexp));
+}
+
+template <class L, bool SHIFT, bool FORCH>
+__device__ __forceinline__ bool split_step_interior(const BufT<double>& in, const BufT<double>& out,
+                                                    const AuxT<double>& A, const Geo& G, const SplitPhys& P, int x,
+                                                    int y) {
+    long long f[9], g[5];
+    uint32_t range = 0u, big = 0u;
+    const SplitCoef c = split_coef(A, G, x, y);
+    split_pull<L>(in, G, P, x, y, f, g, range, big);
+    const bool ok = split_node<SHIFT, FORCH>(f, g, c, P);
+    if (!(ok && fix_ok(range) && big < P.gmax)) return false;
+    split_store(out, G, P, x, y, f, g);
+    return true;
+}
+
+template <class L, bool SHIFT, bool FORCH>
+__device__ __forceinline__ bool split_step_wall(const BufT<double>& in, const BufT<double>& out,
+                                                const AuxT<double>& A, const Geo& G, const SplitPhys& P, int x, int y,
+                                                const WallInfo& w) {
+    long long f[9], g[5], n0ss = 0;
+    uint32_t range = 0u, big = 0u;
+    const int sx = x + w.dx, sy = y + w.dy;
+    const SplitCoef cs = split_coef(A, G, sx, sy), cb = split_coef(A, G, x, y);
+    split_pull<L>(in, G, P, sx, sy, f, g, range, big);
+    if (w.st < 0) {
+        long long o[9];
+        sources<long long>(G, sx + w.dx, sy + w.dy, o);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) n0ss += fix_g(L::ld(in.g + i * G.plane + o[i]), P.gexp, big);
+    }
+    const bool ok = split_wall<SHIFT, FORCH>(f, g, n0ss, cs, cb, w.su, w.st, P);
+    if (!(ok && fix_ok(range) && big < P.gmax)) return false;
+    split_store(out, G, P, x, y, f, g);
+    return true;
+}
+
+// The FP64 path of a node (out of line: it is rarely taken, and its code and
+// registers stay out of the split step's).
+template <class L, bool SHIFT, bool FORCH>
+__device__ __noinline__ void step_node_f64(const BufT<double>* in, const BufT<double>* out, const AuxT<double>* A,
+                                           const KParamsT<double>* K, int x, int y) {
+    step_node<StoreF64T<L>, SHIFT, FORCH>(*in, *out, *A, *K, x, y);
+}
+
 // FP64 step launch shape: threads per block (x extent CLB_F64_BX) and the
-// resident blocks per SM the register allocation is capped for.  Measured
-// at 4096^2 (GB300): 128 threads, 5 blocks (<= 96 registers, 20 warps/SM)
-// 2.98 GLUPS; 256 x 2 blocks 2.97; 6 or 7 blocks of 128 spill and run at
-// 2.88 / 2.96.
+// resident blocks per SM the register allocation is capped for.
 #ifndef CLB_F64_THREADS
 #define CLB_F64_THREADS 128
 #endif
 #ifndef CLB_F64_MINB
-#define CLB_F64_MINB 5
+#define CLB_F64_MINB 4
 #endif
 #ifndef CLB_F64_BX
 #define CLB_F64_BX 64
 #endif
 
 // One launch, two kinds of blocks, so that no warp mixes the interior and
-// the wall path: blocks [0, n_tiles) cover the grid in tiles_x x ... tiles
-// of blockDim nodes and skip wall nodes; the blocks after them take the
-// wall nodes, one per thread, in wall_node order.
-template <class P, bool SHIFT, bool FORCH>
+// the wall path: the first n_wall blocks take the wall nodes, one per thread,
+// in wall_node order (they take longest, so they start first); the others
+// cover the grid in tiles_x x ... tiles of blockDim nodes and skip wall nodes.
+template <bool SHIFT, bool FORCH>
 __global__ void __launch_bounds__(CLB_F64_THREADS, CLB_F64_MINB)
-    k_step(const BufT<typename P::S> in, const BufT<typename P::S> out, const AuxT<typename P::R> A,
-           const KParamsT<typename P::R> K, int tiles_x, int n_tiles) {
-    const int b = blockIdx.x;
-    if (b < n_tiles) {
-        const int x = (b % tiles_x) * blockDim.x + threadIdx.x;
-        const int y = (b / tiles_x) * blockDim.y + threadIdx.y;
+    k_step_f64(const __grid_constant__ BufT<double> in, const __grid_constant__ BufT<double> out,
+               const __grid_constant__ AuxT<double> A, const __grid_constant__ KParamsT<double> K,
+               const __grid_constant__ SplitPhys P, int tiles_x, int n_wall) {
+    int b = blockIdx.x, x, y;
+    if (b >= n_wall) {
+        b -= n_wall;
+        x = (b % tiles_x) * blockDim.x + threadIdx.x;
+        y = (b / tiles_x) * blockDim.y + threadIdx.y;
         if (x >= K.g.nx || y >= K.g.ny) return;
         if ((K.g.wall_x && (x == 0 || x == K.g.nx - 1)) || (K.g.wall_y && (y == 0 || y == K.g.ny - 1))) return;
-        step_interior<P, SHIFT, FORCH>(in, out, A, K, x, y);
+        if (split_step_interior<LdNC, SHIFT, FORCH>(in, out, A, K.g, P, x, y)) return;
     } else {
-        const long long i = (long long)(b - n_tiles) * (blockDim.x * blockDim.y) + threadIdx.y * blockDim.x +
-                            threadIdx.x;
+        const long long i = (long long)b * (blockDim.x * blockDim.y) + threadIdx.y * blockDim.x + threadIdx.x;
         if (i >= wall_count(K.g)) return;
-        int x, y;
         wall_node(K.g, (int)i, x, y);
         WallInfo w;
         wall_info(K.g, K.b, x, y, w);
-        step_wall<P, SHIFT, FORCH>(in, out, A, K, x, y, w);
+        if (split_step_wall<LdNC, SHIFT, FORCH>(in, out, A, K.g, P, x, y, w)) return;
     }
+    step_node_f64<LdNC, SHIFT, FORCH>(&in, &out, &A, &K, x, y);
 }
 
 // FP16 forms, two nodes (x0, x0 + 1) per thread: interior pairs run the
@@ -1529,6 +1615,26 @@ struct CaseT {
     int flip;       // the case's current buffer is b[par ^ flip] (par: the batch's parity)
     int pad_;
 };
+template <>
+struct CaseT<double, double> {
+    KParamsT<double> K;
+    AuxT<double> A;
+    BufT<double> b[2];
+    int flip;
+    int pad_;
+    SplitPhys P;
+};
+
+// One node of a batched FP64 case.
+template <class P, bool SHIFT, bool FORCH>
+__device__ __forceinline__ void step_node_split(const CaseT<double, double>& c, int cur, int x, int y) {
+    using L = typename P::Ld;
+    WallInfo w;
+    const bool done = wall_info(c.K.g, c.K.b, x, y, w)
+                          ? split_step_wall<L, SHIFT, FORCH>(c.b[cur], c.b[1 - cur], c.A, c.K.g, c.P, x, y, w)
+                          : split_step_interior<L, SHIFT, FORCH>(c.b[cur], c.b[1 - cur], c.A, c.K.g, c.P, x, y);
+    if (!done) step_node_f64<L, SHIFT, FORCH>(&c.b[cur], &c.b[1 - cur], &c.A, &c.K, x, y);
+}
 
 // Independent cases advanced together.  `tiles` lists (case, x0, y0) in
 // case order; a block takes the contiguous range [t0, t1), and its threads
@@ -1557,7 +1663,7 @@ __device__ __forceinline__ void batch_tiles(const CaseT<typename P::R, typename 
             if constexpr (NPT == 2)
                 step_pair<P, SHIFT, FORCH>(sc.b[par ^ sc.flip], sc.b[1 - (par ^ sc.flip)], sc.A, sc.K, x, y);
             else
-                step_node<P, SHIFT, FORCH>(sc.b[par ^ sc.flip], sc.b[1 - (par ^ sc.flip)], sc.A, sc.K, x, y);
+                step_node_split<P, SHIFT, FORCH>(sc, par ^ sc.flip, x, y);
         }
     }
 }
@@ -1856,6 +1962,19 @@ __global__ void k_coef(const double* __restrict__ phi, const double* __restrict_
     c.hgb = hp * gbeta;
     c.hgy = hp * ayg[i / nx];
     coef[i] = c;
+}
+
+// The same constants as split numbers, in planes (see SplitCoef).
+__global__ void k_split_coef(const CoefT<double>* __restrict__ coef, float2* __restrict__ out, long long n) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const CoefT<double> c = coef[i];
+    const double v[kSplitPlanes] = {c.ip, c.l0, c.l0sq, c.aux, c.hdar, c.hgx, c.hgb, c.hgy};
+#pragma unroll
+    for (int k = 0; k < kSplitPlanes; ++k) {
+        const sf s = sf_make(v[k]);
+        out[k * n + i] = make_float2(s.h, s.l);
+    }
 }
 
 // FP32 porosity (dense) for the FP16 rest-shifted form, or FP32 1/phi
