@@ -325,6 +325,22 @@ static void free_all(clb_handle* h) {
 }
 
 // ------------------------------------------------------------------ kernels
+// Launch that may start before the kernel in front of it has ended; the
+// kernel itself waits for it (pdl_begin).
+template <class... P, class... V>
+static void launch_pdl(void (*k)(P...), unsigned grid, dim3 block, cudaStream_t s, const V&... v) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, P(v)...);   // an error stays for the caller's cudaGetLastError
+}
+
 static void step_f64(clb_handle* h, cudaStream_t s) {
     const BufT<double> in = h->buf<double>(h->par), out = h->buf<double>(1 - h->par);
     const AuxT<double> A = h->aux64();
@@ -334,10 +350,10 @@ static void step_f64(clb_handle* h, cudaStream_t s) {
     const int threads = (int)(h->block.x * h->block.y);
     const int tx = (int)h->grid.x, nw = (int)((wall_count(K.g) + threads - 1) / threads);
     const unsigned nb = (unsigned)nw + h->grid.x * h->grid.y;
-    if (sh && fo) k_step_f64<true, true><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
-    else if (sh) k_step_f64<true, false><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
-    else if (fo) k_step_f64<false, true><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
-    else k_step_f64<false, false><<<nb, h->block, 0, s>>>(in, out, A, K, h->sp, tx, nw);
+    if (sh && fo) launch_pdl(k_step_f64<true, true>, nb, h->block, s, in, out, A, K, h->sp, tx, nw);
+    else if (sh) launch_pdl(k_step_f64<true, false>, nb, h->block, s, in, out, A, K, h->sp, tx, nw);
+    else if (fo) launch_pdl(k_step_f64<false, true>, nb, h->block, s, in, out, A, K, h->sp, tx, nw);
+    else launch_pdl(k_step_f64<false, false>, nb, h->block, s, in, out, A, K, h->sp, tx, nw);
 }
 
 // FP16 forms: two nodes per thread (k_step2), grid over node pairs.
@@ -353,7 +369,7 @@ static void step2_as(clb_handle* h, cudaStream_t s, long long limit = TT_LIMIT, 
     const Geo& G = h->k32.g;
     const int tx = (int)h->grid2.x;
     int nt = (int)(h->grid2.x * h->grid2.y), outer = 0;
-    if constexpr (std::is_same<P, StoreH16N>::value) {
+    if constexpr (std::is_same<P, StoreH16NT<LdPD>>::value) {
         if (h->tma) {
             const int b = h->par;
             const dim3 gr((unsigned)h->tma_grid), bl(TT_THREADS);
@@ -377,21 +393,21 @@ static void step2_as(clb_handle* h, cudaStream_t s, long long limit = TT_LIMIT, 
     const unsigned nb = (unsigned)(nt + (edge_count(G) + threads - 1) / threads);
     if (nb == 0) return;
     if (outer) {
-        if (sh && fo) k_step2<P, true, true, true><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
-        else if (sh) k_step2<P, true, false, true><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
-        else if (fo) k_step2<P, false, true, true><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
-        else k_step2<P, false, false, true><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
+        if (sh && fo) launch_pdl(k_step2<P, true, true, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
+        else if (sh) launch_pdl(k_step2<P, true, false, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
+        else if (fo) launch_pdl(k_step2<P, false, true, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
+        else launch_pdl(k_step2<P, false, false, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
     } else {
-        if (sh && fo) k_step2<P, true, true><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
-        else if (sh) k_step2<P, true, false><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
-        else if (fo) k_step2<P, false, true><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
-        else k_step2<P, false, false><<<nb, h->block2, 0, s>>>(in, out, A, h->k32, tx, nt);
+        if (sh && fo) launch_pdl(k_step2<P, true, true, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
+        else if (sh) launch_pdl(k_step2<P, true, false, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
+        else if (fo) launch_pdl(k_step2<P, false, true, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
+        else launch_pdl(k_step2<P, false, false, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
     }
 }
 
 static void launch_step(clb_handle* h, cudaStream_t s) {
-    if (h->prec == CLB_F16S) step2_as<StoreH16>(h, s);
-    else if (h->prec == CLB_F16N) step2_as<StoreH16N>(h, s);
+    if (h->prec == CLB_F16S) step2_as<StoreH16T<LdPD>>(h, s);
+    else if (h->prec == CLB_F16N) step2_as<StoreH16NT<LdPD>>(h, s);
     else step_f64(h, s);
     h->par = 1 - h->par;
 }
@@ -890,7 +906,7 @@ extern "C" int clb_tma_selftest(clb_handle* h, int64_t limit_cycles) {
     CK(h, cudaStreamSynchronize(h->stream));
     const bool save = h->tma;
     h->tma = true;
-    step2_as<StoreH16N>(h, h->stream, (long long)limit_cycles, 1);   // writes the idle buffer; time and parity unchanged
+    step2_as<StoreH16NT<LdPD>>(h, h->stream, (long long)limit_cycles, 1);   // writes the idle buffer; time and parity unchanged
     h->tma = save;
     CK(h, cudaGetLastError());
     CK(h, cudaStreamSynchronize(h->stream));

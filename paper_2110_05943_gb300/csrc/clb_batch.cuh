@@ -43,6 +43,12 @@ struct clb_batch {
     bool graph_failed = false;
     int mode = CLB_BATCH_GRAPH;   // measured faster on the 512-case workload (FP16N 30.8 vs 30.1 GLUPS)
     GridBarrier* bar = nullptr;     // persistent mode: grid barrier state (device)
+    // Nusselt numbers of all cases: (L, dT) per case, results, current buffers
+    double2* geom = nullptr;
+    double* nu = nullptr;           // device, then its pinned copy
+    double* nu_host = nullptr;
+    int* cur = nullptr;             // device, then its pinned source
+    int* cur_host = nullptr;
     int pgrid = 0;                  // persistent mode: resident blocks of the launch
     long long wait_limit = 4000000000LL;   // barrier wait bound, SM cycles (~2 s)
     std::string err;
@@ -187,10 +193,10 @@ static void batch_launch_as(clb_batch* b, cudaStream_t s, cudaStream_t side) {
             const unsigned g = (unsigned)b->n_work;
             const int4 *w = b->work, *t = b->itiles, *e = b->echunks;
             const int n = b->n_itiles, pc = b->per_cta, par = b->par;
-            if (b->shift && b->forch) k_step_batch_mix<P, true, true><<<g, block, 0, s>>>(tab, w, t, n, pc, e, par);
-            else if (b->shift) k_step_batch_mix<P, true, false><<<g, block, 0, s>>>(tab, w, t, n, pc, e, par);
-            else if (b->forch) k_step_batch_mix<P, false, true><<<g, block, 0, s>>>(tab, w, t, n, pc, e, par);
-            else k_step_batch_mix<P, false, false><<<g, block, 0, s>>>(tab, w, t, n, pc, e, par);
+            if (b->shift && b->forch) launch_pdl(k_step_batch_mix<P, true, true>, g, block, s, tab, w, t, n, pc, e, par);
+            else if (b->shift) launch_pdl(k_step_batch_mix<P, true, false>, g, block, s, tab, w, t, n, pc, e, par);
+            else if (b->forch) launch_pdl(k_step_batch_mix<P, false, true>, g, block, s, tab, w, t, n, pc, e, par);
+            else launch_pdl(k_step_batch_mix<P, false, false>, g, block, s, tab, w, t, n, pc, e, par);
             return;
         }
         const bool fork = side && b->n_itiles > 0 && b->n_echunks > 0;
@@ -219,10 +225,10 @@ static void batch_launch_as(clb_batch* b, cudaStream_t s, cudaStream_t side) {
         }
     } else {
         const int grid = (b->ntiles + b->per_cta - 1) / b->per_cta;
-        if (b->shift && b->forch) k_step_batch<P, NPT, true, true><<<grid, block, 0, s>>>(tab, b->tiles, b->ntiles, b->per_cta, b->par);
-        else if (b->shift) k_step_batch<P, NPT, true, false><<<grid, block, 0, s>>>(tab, b->tiles, b->ntiles, b->per_cta, b->par);
-        else if (b->forch) k_step_batch<P, NPT, false, true><<<grid, block, 0, s>>>(tab, b->tiles, b->ntiles, b->per_cta, b->par);
-        else k_step_batch<P, NPT, false, false><<<grid, block, 0, s>>>(tab, b->tiles, b->ntiles, b->per_cta, b->par);
+        if (b->shift && b->forch) launch_pdl(k_step_batch<P, NPT, true, true>, (unsigned)grid, block, s, tab, b->tiles, b->ntiles, b->per_cta, b->par);
+        else if (b->shift) launch_pdl(k_step_batch<P, NPT, true, false>, (unsigned)grid, block, s, tab, b->tiles, b->ntiles, b->per_cta, b->par);
+        else if (b->forch) launch_pdl(k_step_batch<P, NPT, false, true>, (unsigned)grid, block, s, tab, b->tiles, b->ntiles, b->per_cta, b->par);
+        else launch_pdl(k_step_batch<P, NPT, false, false>, (unsigned)grid, block, s, tab, b->tiles, b->ntiles, b->per_cta, b->par);
     }
 }
 
@@ -277,9 +283,9 @@ static cudaError_t batch_persist(clb_batch* b, cudaStream_t s, int par0, int nst
 
 static void batch_launch(clb_batch* b, cudaStream_t s, cudaStream_t side = nullptr) {
     if (b->ntiles > 0) {
-        if (b->prec == CLB_F16S) batch_launch_as<StoreH16, 2>(b, s, side);
-        else if (b->prec == CLB_F16N) batch_launch_as<StoreH16N, 2>(b, s, side);
-        else batch_launch_as<StoreF64, 1>(b, s, side);
+        if (b->prec == CLB_F16S) batch_launch_as<StoreH16T<LdPD>, 2>(b, s, side);
+        else if (b->prec == CLB_F16N) batch_launch_as<StoreH16NT<LdPD>, 2>(b, s, side);
+        else batch_launch_as<StoreF64T<LdPD>, 1>(b, s, side);
     }
     b->par = 1 - b->par;
 }
@@ -409,6 +415,16 @@ extern "C" int clb_batch_init(clb_batch** out, int32_t ncase, const clb_params* 
         bfail(b, CLB_ERR_CUDA, "clb_batch_init: grid barrier allocation failed");
         return bail(CLB_ERR_CUDA);
     }
+    std::vector<double2> geom(ncase);
+    for (int c = 0; c < ncase; ++c) geom[c] = make_double2(b->cases[c]->lat.L, p[c].dT);
+    if (cudaMalloc(&b->geom, ncase * sizeof(double2)) != cudaSuccess ||
+        cudaMemcpy(b->geom, geom.data(), ncase * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMalloc(&b->nu, ncase * sizeof(double)) != cudaSuccess || cudaMalloc(&b->cur, ncase * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&b->nu_host, ncase * sizeof(double)) != cudaSuccess ||
+        cudaMallocHost(&b->cur_host, ncase * sizeof(int)) != cudaSuccess) {
+        bfail(b, CLB_ERR_OOM, "clb_batch_init: reduction buffers");
+        return bail(CLB_ERR_OOM);
+    }
     const int rc = batch_build_tiles(b);
     if (rc != CLB_OK) return bail(rc);
     *out = b;
@@ -510,15 +526,40 @@ extern "C" int clb_batch_set_active(clb_batch* b, const int32_t* active) {
     return batch_build_tiles(b);
 }
 
+template <class P>
+static void batch_nusselt_as(clb_batch* b, int side) {
+    k_nusselt_batch<P><<<(unsigned)b->cases.size(), kRedThreads, 0, b->stream>>>(
+        (const CaseT<typename P::R, typename P::S>*)b->table, b->cur, b->geom, side, b->nu);
+}
+
 extern "C" int clb_batch_nusselt(clb_batch* b, int32_t side, double* nu) {
     if (!b || !nu) return CLB_ERR_ARG;
     const int rb = batch_check(b);
     if (rb != CLB_OK) return rb;
     batch_sync_cases(b);
-    for (size_t c = 0; c < b->cases.size(); ++c) {
-        const int rc = clb_nusselt(b->cases[c], side, &nu[c]);
-        if (rc != CLB_OK) return bfail(b, rc, "clb_batch_nusselt: case %zu: %s", c, b->cases[c]->err.c_str());
+    if (side < 0 || side > 3) return bfail(b, CLB_ERR_ARG, "clb_batch_nusselt: case 0: clb_nusselt: side must be 0..3");
+    const size_t nc = b->cases.size();
+    size_t bad = nc;   // the first case whose grid has no such number; the cases before it are still given
+    for (size_t c = 0; c < nc; ++c) {
+        const clb_params& p = b->cases[c]->prm;
+        b->cur_host[c] = b->cases[c]->par;
+        if (bad == nc && ((side < 2 ? p.ny : p.nx) < 2 || (side < 2 ? p.nx : p.ny) < 3)) bad = c;
     }
+    if (bad > 0) {
+        CKB(b, cudaMemcpyAsync(b->cur, b->cur_host, nc * sizeof(int), cudaMemcpyHostToDevice, b->stream));
+        if (b->prec == CLB_F16S) batch_nusselt_as<StoreH16>(b, side);
+        else if (b->prec == CLB_F16N) batch_nusselt_as<StoreH16N>(b, side);
+        else batch_nusselt_as<StoreF64>(b, side);
+        CKB(b, cudaGetLastError());
+        CKB(b, cudaMemcpyAsync(b->nu_host, b->nu, nc * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+        CKB(b, cudaStreamSynchronize(b->stream));
+    }
+    for (size_t c = 0; c < bad; ++c) {
+        nu[c] = b->nu_host[c];
+        if (!std::isfinite(nu[c]))
+            return bfail(b, CLB_ERR_UNSTABLE, "clb_batch_nusselt: case %zu: clb_nusselt: non-finite result", c);
+    }
+    if (bad < nc) return bfail(b, CLB_ERR_ARG, "clb_batch_nusselt: case %zu: clb_nusselt: grid too small", bad);
     return CLB_OK;
 }
 
@@ -597,6 +638,11 @@ extern "C" void clb_batch_destroy(clb_batch* b) {
     batch_drop_graphs(b);
     for (clb_handle* h : b->cases) clb_destroy(h);
     cudaFree(b->bar);
+    cudaFree(b->geom);
+    cudaFree(b->nu);
+    cudaFree(b->cur);
+    if (b->nu_host) cudaFreeHost(b->nu_host);
+    if (b->cur_host) cudaFreeHost(b->cur_host);
     cudaFree(b->table);
     cudaFree(b->tiles);
     cudaFree(b->itiles);

