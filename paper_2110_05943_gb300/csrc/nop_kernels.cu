@@ -11,6 +11,8 @@
 //   dgrad   : dX[p, ci]  = sum_{tap, co} dY[p - d(tap), co] W[tap, ci, co]
 //   wgrad   : dW[tap, ci, co] += sum_p X[p + d(tap), ci] dY[p, co]   (split K, FP32 atomics)
 // In order of preference (the first that takes the shape runs):
+//   k_conv_row / k_wgrad_row -- image rows kept in a ring in shared memory, each
+//     fetched once for all nine taps (padded channels: 32 in, multiples of 32);
 //   k_conv_tma / k_wgrad_tma -- operands brought by TMA from the NHWC tensors
 //     into swizzled shared memory, tcgen05.mma with the accumulator in TMEM
 //     (whole-row pixel tiles, channel counts multiples of 8);
@@ -475,18 +477,18 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __nv_bfloat16* __r
 // land in shared memory as 2 kc-byte rows with the matching swizzle (64 or
 // 128 bytes), the K-major layout tcgen05.mma reads (K = 16 per MMA: the
 // descriptor start advances 32 bytes).
-//   warp 4 (one thread): producer -- a ring of `stages` buffers; each stage's
+//   warp 8 (one thread): producer -- a ring of `stages` buffers; each stage's
 //     "full" mbarrier expects the bytes of both boxes;
-//   warp 5 (one thread): MMA issuer -- kc / 16 MMAs per stage, committed to
+//   warp 9 (one thread): MMA issuer -- kc / 16 MMAs per stage, committed to
 //     the stage's "empty" mbarrier; the tile's accumulator alternates between
 //     two TMEM buffers, committed to that buffer's "acc_full" mbarrier;
-//   warps 0-3: epilogue -- warp w reads TMEM lanes 32w .. 32w + 31 (one pixel
-//     per thread) of the finished buffer, adds the bias, applies ReLU or the
+//   warps 0-3 and 4-7: epilogue of the two buffers -- warp w reads TMEM lanes
+//     32 (w mod 4) .. + 31 (one pixel per thread) of its finished buffer, adds the bias, applies ReLU or the
 //     mask, stores, and releases the buffer ("acc_empty", 128 arrivals), so
 //     the next tile's MMAs overlap this tile's epilogue.
 // Every wait is bounded; on expiry a role stops, the CTA waits (bounded) for
 // the loads and MMAs it issued, frees its TMEM and sets the flag.
-constexpr int TM_THREADS = 192;
+constexpr int TM_THREADS = 320;
 // Most stages of the copy rings (build-time options).  Shallower rings leave
 // shared memory for the weight gradients, which run concurrently on a side
 // stream during training: 5 and 3 measured 1.28 ms per training step against
@@ -496,6 +498,15 @@ constexpr int TM_THREADS = 192;
 #endif
 #ifndef CLB_WG_MAX_STAGES
 #define CLB_WG_MAX_STAGES 3
+#endif
+#ifndef CLB_ROW_MAX_STAGES
+#define CLB_ROW_MAX_STAGES 6
+#endif
+#ifndef CLB_WR_MAX_STAGES
+#define CLB_WR_MAX_STAGES 5
+#endif
+#ifndef CLB_WR_CTAS
+#define CLB_WR_CTAS 1
 #endif
 constexpr int TM_BIAS_MAX = 1024;                // outputs whose bias is staged in shared memory
 
@@ -531,27 +542,44 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
 
 // Bounded wait with mbarrier.try_wait (the hardware may suspend the thread
 // between tries, so idle threads cost little issue bandwidth).
-__device__ __forceinline__ bool mbar_wait_try(uint32_t a, uint32_t parity, long long limit) {
-    const long long t0 = clock64();
-    while (true) {
-        uint32_t done;
-        asm volatile(
-            "{\n .reg .pred P;\n mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n selp.u32 %0, 1, 0, P;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if (clock64() - t0 > limit) return false;
-    }
+// One try_wait, suspended for at most 64 ns (the default bound is longer, and
+// a weight gradient took 2 us more with it).
+__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred P;\n mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2, 64;\n selp.u32 %0, 1, 0, P;\n}\n"
+        : "=r"(done)
+        : "r"(a), "r"(parity)
+        : "memory");
+    return done;
 }
 
-// Shared-memory descriptor of a K-major operand stored as R-byte rows with
-// the R-byte swizzle (R = 128 or 64): 8-row groups 8R bytes apart (stride
-// byte offset), descriptor version 1, swizzle mode 2 (128-byte) or 4 (64-byte).
-__device__ __forceinline__ uint64_t tc_desc_sw(uint32_t addr, int row_bytes) {
-    const uint64_t mode = row_bytes == 128 ? 2ull : 4ull;
-    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)((8 * row_bytes) >> 4) << 32) |
-           (1ull << 46) | (mode << 61);
+__device__ __forceinline__ bool mbar_wait_try(uint32_t a, uint32_t parity, long long limit) {
+    if (mbar_try(a, parity)) return true;   // the usual case, without reading the clock
+    const long long t0 = clock64();
+    while (!mbar_try(a, parity))
+        if (clock64() - t0 > limit) return mbar_try(a, parity);
+    return true;
+}
+
+// The MMA-issuing thread is one thread: what it computes per MMA adds to the
+// tile's chain (an MMA of M 128, K 16 with at most 64 outputs takes 45-48 cycles
+// issued back to back, ~200 with each descriptor built from its address).  A
+// shared-memory descriptor of a swizzled operand (rows of row_bytes = 128 or 64,
+// 8-row groups 8 row_bytes apart, descriptor version 1, swizzle mode 2 or 4) has
+// a constant upper word, and its lower word moves with the address / 16: the
+// loops below only add to 32-bit words.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | ((lbo >> 4) << 16); }
+__device__ __forceinline__ constexpr uint32_t desc_hi(int row_bytes) {
+    return (uint32_t)((8 * row_bytes) >> 4) | (1u << 14) | ((row_bytes == 128 ? 2u : 4u) << 29);
+}
+__device__ __forceinline__ void tc_mma_lo(uint32_t tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                          uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b64 a, b;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n setp.ne.b32 p, %6, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(tmem),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc)
+        : "memory");
 }
 
 // 32 consecutive accumulator columns of this thread's TMEM lane (no wait).
@@ -613,6 +641,62 @@ __device__ __forceinline__ void tm_store8(const uint32_t* r, int o, int c0, int 
     }
 }
 
+// The same for whole groups of 32 BF16 outputs with 16-byte stores, the case
+// of every padded layer: no per-element tests, the bias as 16-byte shared
+// loads, the mask read before the accumulator is waited for (mk, 32 outputs
+// from c0 = 0) and applied to BF16 pairs.  FP32 sums and their rounding as in
+// tm_store8; about 150 instructions per 32 outputs against 600.
+__device__ __forceinline__ void tm_mask_load(const __nv_bfloat16* __restrict__ mask, int o, uint4 (&mk)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mk[q] = __ldg(reinterpret_cast<const uint4*>(mask + o) + q);
+}
+// v where m > 0 (BF16 pairs; NaN counts as not greater), else 0
+__device__ __forceinline__ uint32_t tm_masked(uint32_t v, uint32_t m) {
+    const __nv_bfloat162 z = __floats2bfloat162_rn(0.0f, 0.0f);
+    return v & __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&m), z);
+}
+__device__ __forceinline__ void tm_store_row32(uint32_t taddr, int o, int nt, const float* sb,
+                                               const __nv_bfloat16* __restrict__ mask, uint4 (&mk)[4],
+                                               __nv_bfloat16* __restrict__ out, int relu) {
+    for (int c0 = 0; c0 < nt; c0 += 32) {
+        uint32_t r[32];
+        tc_ld32_nowait(taddr + (uint32_t)c0, r);
+        if (mask && c0 > 0) tm_mask_load(mask, o + c0, mk);
+        tc_wait_ld();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[8 * q + j]);
+            if (sb) {
+                const float4 b0 = *reinterpret_cast<const float4*>(sb + c0 + 8 * q), b1 = *reinterpret_cast<const float4*>(sb + c0 + 8 * q + 4);
+                v[0] += b0.x;
+                v[1] += b0.y;
+                v[2] += b0.z;
+                v[3] += b0.w;
+                v[4] += b1.x;
+                v[5] += b1.y;
+                v[6] += b1.z;
+                v[7] += b1.w;
+            }
+            if (relu)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = fmaxf(v[j], 0.0f);
+            uint4 pk;
+            __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(&pk);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) h2[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+            if (mask) {
+                pk.x = tm_masked(pk.x, mk[q].x);
+                pk.y = tm_masked(pk.y, mk[q].y);
+                pk.z = tm_masked(pk.z, mk[q].z);
+                pk.w = tm_masked(pk.w, mk[q].w);
+            }
+            *reinterpret_cast<uint4*>(out + o + c0 + 8 * q) = pk;
+        }
+    }
+}
+
 // Epilogue of one accumulator row (pixel `row`, outputs n0 .. n0 + nt - 1):
 // 32 columns per TMEM load and wait, then the rest 8 at a time.
 __device__ __forceinline__ void tm_store_row(uint32_t taddr, int row, int n0, int nt, int tile_n, int N,
@@ -639,18 +723,18 @@ __device__ __forceinline__ void tm_store_row(uint32_t taddr, int row, int n0, in
 // (cin, taps, cout).  MODE DGRAD: A = output gradient dY (C = cout) at the
 // mirrored taps, B = W [taps * cin][cout] viewed as (cout, cin, taps).
 // tmem_cols: columns of one accumulator buffer (two are allocated).
-template <int MODE>
-__global__ void __launch_bounds__(TM_THREADS, 1) k_conv_tma(const __grid_constant__ CUtensorMap mapA,
+template <int MODE, int kc>
+__global__ void __launch_bounds__(TM_THREADS, 2) k_conv_tma(const __grid_constant__ CUtensorMap mapA,
                                                          const __grid_constant__ CUtensorMap mapB,
                                                          const float* __restrict__ bias,
                                                          const __nv_bfloat16* __restrict__ mask, void* __restrict__ out,
                                                          int out_f32, int relu, ConvShape s, int M, int N, int tile_n,
-                                                         int tmem_cols, int vec_out, int stages, int cchunks, int kc,
+                                                         int tmem_cols, int vec_out, int stages, int cchunks,
                                                          int ntiles, int ntn) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* const smem =
         smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // swizzled tiles start on 1024 B
-    __shared__ float s_bias[TM_BIAS_MAX];                               // the bias of all N outputs
+    __shared__ __align__(16) float s_bias[TM_BIAS_MAX];                               // the bias of all N outputs
     const int a_bytes = TC_M * kc * 2, b_bytes = tile_n * kc * 2;
     const int stage_bytes = a_bytes + b_bytes;                           // a multiple of 1024 (tile_n % 16 == 0)
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + stages * stage_bytes);
@@ -666,7 +750,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) k_conv_tma(const __grid_constan
     const int niter = s.taps * cchunks;
     const int hw = s.h * s.w;
 
-    if (warp == 4) {
+    if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(2 * tmem_cols)
                      : "memory");
@@ -694,35 +778,37 @@ __global__ void __launch_bounds__(TM_THREADS, 1) k_conv_tma(const __grid_constan
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
+    const uint32_t fb0 = smem_u32(full), eb = smem_u32(empty), ring = smem_u32(smem), ring_lo = desc_lo(ring, 16);
     bool ok = true;
-    if (warp == 4) {
+    if (warp == 8) {
         if (lane == 0) {   // producer
             int it = 0, st = 0, ph = 0;   // global iteration, its stage and the stage's use count parity
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
                 const int m0 = (t / ntn) * TC_M, n0 = (t % ntn) * tile_n;
                 const int img = m0 / hw, rem = m0 - img * hw, h0 = rem / s.w, w0 = rem - h0 * s.w;
-                for (int j = 0; j < niter; ++j) {
-                    if (it >= stages && !mbar_wait_try(smem_u32(&empty[st]), ph ^ 1, TC_TIMEOUT_CYCLES)) {
-                        ok = false;
-                        break;
-                    }
-                    const int tap = j / cchunks, c0 = (j - tap * cchunks) * kc;
-                    const int ddy = sg * tap_dy(tap, s.taps), ddx = sg * tap_dx(tap, s.taps);
-                    const uint32_t fb = smem_u32(&full[st]), a_dst = smem_u32(smem + st * stage_bytes);
-                    mbar_expect_tx(fb, (uint32_t)stage_bytes);
-                    tma_load_4d(a_dst, &mapA, fb, c0, w0 + ddx, h0 + ddy, img);
-                    if (MODE == FWD) tma_load_3d(a_dst + a_bytes, &mapB, fb, c0, tap, n0);
-                    else tma_load_3d(a_dst + a_bytes, &mapB, fb, c0, n0, tap);
-                    ++it;
-                    if (++st == stages) {
-                        st = 0;
-                        ph ^= 1;
+                for (int tap = 0; tap < s.taps && ok; ++tap) {
+                    const int ax = w0 + sg * tap_dx(tap, s.taps), ay = h0 + sg * tap_dy(tap, s.taps);
+                    for (int c0 = 0; c0 < cchunks * kc; c0 += kc) {
+                        if (it >= stages && !mbar_wait_try(eb + 8 * st, ph ^ 1, TC_TIMEOUT_CYCLES)) {
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t fb = fb0 + 8 * st, a_dst = ring + st * stage_bytes;
+                        mbar_expect_tx(fb, (uint32_t)stage_bytes);
+                        tma_load_4d(a_dst, &mapA, fb, c0, ax, ay, img);
+                        if (MODE == FWD) tma_load_3d(a_dst + a_bytes, &mapB, fb, c0, tap, n0);
+                        else tma_load_3d(a_dst + a_bytes, &mapB, fb, c0, n0, tap);
+                        ++it;
+                        if (++st == stages) {
+                            st = 0;
+                            ph ^= 1;
+                        }
                     }
                 }
             }
             s_issued = it;
         }
-    } else if (warp == 5) {
+    } else if (warp == 9) {
         if (lane == 0) {   // MMA issuer
             const uint32_t idesc = tc_idesc(tile_n);
             int it = 0, st = 0, ph = 0, lt = 0;
@@ -735,16 +821,17 @@ __global__ void __launch_bounds__(TM_THREADS, 1) k_conv_tma(const __grid_constan
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d = tmem + (uint32_t)(b * tmem_cols);
                 for (int j = 0; j < niter; ++j) {
-                    if (!mbar_wait_try(smem_u32(&full[st]), ph, TC_TIMEOUT_CYCLES)) {
+                    if (!mbar_wait_try(fb0 + 8 * st, ph, TC_TIMEOUT_CYCLES)) {
                         ok = false;
                         break;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a0 = smem_u32(smem + st * stage_bytes), b0 = a0 + a_bytes;
+                    const uint32_t al = ring_lo + (uint32_t)(st * (stage_bytes >> 4)), bl = al + (uint32_t)(a_bytes >> 4);
+#pragma unroll
                     for (int ks = 0; ks < kc / 16; ++ks)
-                        tc_mma(d, tc_desc_sw(a0 + ks * 32, 2 * kc), tc_desc_sw(b0 + ks * 32, 2 * kc), idesc,
-                               (j > 0 || ks > 0) ? 1u : 0u);
-                    tc_commit(smem_u32(&empty[st]));
+                        tc_mma_lo(d, al + 2 * ks, desc_hi(2 * kc), bl + 2 * ks, desc_hi(2 * kc), idesc,
+                                  ks > 0 ? 1u : (uint32_t)(j > 0));
+                    tc_commit(eb + 8 * st);
                     ++it;
                     if (++st == stages) {
                         st = 0;
@@ -756,27 +843,33 @@ __global__ void __launch_bounds__(TM_THREADS, 1) k_conv_tma(const __grid_constan
             s_consumed = it;
             tc_commit(smem_u32(done));   // arrives once every MMA issued above has completed
         }
-    } else {   // epilogue: warps 0-3
-        int lt = 0;
-        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+    } else {   // epilogue: warps 0-3 the even tiles (accumulator 0), warps 4-7 the odd ones
+        const int quad = warp & 3;
+        const bool fast = !out_f32 && vec_out && N % tile_n == 0 && tile_n % 32 == 0 && (sbias || !bias);
+        for (int lt = warp >> 2, t = blockIdx.x + lt * gridDim.x; t < ntiles; t += 2 * gridDim.x, lt += 2) {
             const int b = lt & 1;
+            const int m0 = (t / ntn) * TC_M, n0 = (t % ntn) * tile_n;
+            const int row = m0 + quad * 32 + lane;
+            uint4 mk[4];
+            if (fast && mask) tm_mask_load(mask, row * N + n0, mk);
             if (!mbar_wait_try(smem_u32(&acc_full[b]), (lt >> 1) & 1, TC_TIMEOUT_CYCLES)) {
                 ok = false;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int m0 = (t / ntn) * TC_M, n0 = (t % ntn) * tile_n;
-            const int row = m0 + warp * 32 + lane;
-            tm_store_row(tmem + (uint32_t)(b * tmem_cols) + ((uint32_t)(warp * 32) << 16), row, n0,
+            if (fast)
+                tm_store_row32(tmem + (uint32_t)(b * tmem_cols) + ((uint32_t)(quad * 32) << 16), row * N + n0, tile_n,
+                               sbias ? s_bias + n0 : nullptr, mask, mk, reinterpret_cast<__nv_bfloat16*>(out), relu);
+            else tm_store_row(tmem + (uint32_t)(b * tmem_cols) + ((uint32_t)(quad * 32) << 16), row, n0,
                          min(tile_n, N - n0), tile_n, N, sbias ? s_bias + n0 : (bias ? bias + n0 : nullptr), mask, out, out_f32, relu,
                          vec_out);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(smem_u32(&acc_empty[b]));
         }
     }
-    if (tid == 160) ok = mbar_wait_try(smem_u32(done), 0u, TC_TIMEOUT_CYCLES) && ok;
+    if (tid == 288) ok = mbar_wait_try(smem_u32(done), 0u, TC_TIMEOUT_CYCLES) && ok;
     ok = __syncthreads_and(ok);
-    if (!ok && tid == 128) {
+    if (!ok && tid == 256) {
         // loads still in flight write this CTA's shared memory: wait for them (bounded)
         for (int it = s_consumed; it < s_issued; ++it)
             mbar_wait_try(smem_u32(&full[it % stages]), (it / stages) & 1, TC_TIMEOUT_CYCLES);
@@ -784,7 +877,200 @@ __global__ void __launch_bounds__(TM_THREADS, 1) k_conv_tma(const __grid_constan
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 4)
+    if (warp == 8)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * tmem_cols)
+                     : "memory");
+}
+
+// ---------------------------------------------------------------- row-ring convolution
+// Forward and input gradient of 3x3 layers with 32 (padded) input channels on
+// images whose width is a multiple of 128: k_conv_tma fetches every pixel once per tap (nine boxes per 128-pixel
+// tile), and those copies' request rate, not the MMAs, set its pace.  Here a
+// CTA walks down the image: each 128-pixel row segment is fetched once, with
+// one pixel of halo on either side, into a ring of `stages`; the tile of row y
+// takes its nine taps from the three newest rows.  A tap's dx only moves the
+// start of the K-major operand by one pixel's bytes (the swizzle follows the
+// address).  All weights stay in shared memory.  Same products in the same
+// order as k_conv_tma (taps, then channels): the same bits.  Roles, TMEM
+// double buffering and bounded waits as there.
+template <int MODE>
+__global__ void __launch_bounds__(TM_THREADS, 2)
+    k_conv_row(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+               const float* __restrict__ bias, const __nv_bfloat16* __restrict__ mask, void* __restrict__ out, int out_f32,
+               int relu, ConvShape s, int N, int tile_n, int tmem_cols, int vec_out, int stages, int a_bytes, int total) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* const wsm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // weights, then the ring
+    __shared__ __align__(16) float s_bias[TM_BIAS_MAX];
+    constexpr int kc = 32, rb = kc * 2;                                  // channels, and bytes per pixel
+    const int b_bytes = tile_n * kc * 2, stage_bytes = a_bytes;
+    unsigned char* const smem = wsm + 9 * b_bytes;
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + stages * stage_bytes);
+    uint64_t* empty = full + stages;
+    uint64_t* acc_full = empty + stages;                                 // [2]
+    uint64_t* acc_empty = acc_full + 2;                                  // [2]
+    uint64_t* wfull = acc_empty + 2;
+    uint64_t* done = wfull + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    __shared__ int s_issued, s_consumed;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int segs = s.w / TC_M;
+    const int t0 = (int)((long long)total * blockIdx.x / gridDim.x), t1 = (int)((long long)total * (blockIdx.x + 1) / gridDim.x);
+
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(2 * tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(smem_u32(&full[i]));
+            mbar_init(smem_u32(&empty[i]));
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&acc_full[b]));
+            mbar_init_n(smem_u32(&acc_empty[b]), 128);
+        }
+        mbar_init(smem_u32(wfull));
+        mbar_init(smem_u32(done));
+        s_issued = 0;
+        s_consumed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const bool sbias = bias && N <= TM_BIAS_MAX;
+    if (sbias)
+        for (int i = tid; i < N; i += TM_THREADS) s_bias[i] = bias[i];
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+
+    // Rows are numbered (image, segment, y), y fastest; a run stays within one
+    // image and segment and needs the rows ya - 1 .. yb.
+    bool ok = true, weights = false;
+    if (warp == 8) {
+        if (lane == 0) {   // producer
+            const uint32_t wb = smem_u32(wfull);
+            mbar_expect_tx(wb, (uint32_t)(9 * b_bytes));
+            for (int tap = 0; tap < 9; ++tap) {
+                const uint32_t dst = smem_u32(wsm) + (uint32_t)(tap * b_bytes);
+                if (MODE == FWD) tma_load_3d(dst, &mapB, wb, 0, tap, 0);
+                else tma_load_3d(dst, &mapB, wb, 0, 0, tap);
+            }
+            int it = 0, st = 0, ph = 0;
+            for (int t = t0; t < t1 && ok;) {
+                const int is = t / s.h, ya = t - is * s.h, yb = min(s.h, ya + (t1 - t));
+                const int img = is / segs, w0 = (is - img * segs) * TC_M;
+                for (int x = ya - 1; x <= yb; ++x) {
+                    if (it >= stages && !mbar_wait_try(smem_u32(&empty[st]), ph ^ 1, TC_TIMEOUT_CYCLES)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t fb = smem_u32(&full[st]), base = smem_u32(smem + st * stage_bytes);
+                    mbar_expect_tx(fb, (uint32_t)((TC_M + 2) * rb));
+                    tma_load_4d(base, &mapA, fb, 0, w0 - 1, x, img);
+                    ++it;
+                    if (++st == stages) {
+                        st = 0;
+                        ph ^= 1;
+                    }
+                }
+                t += yb - ya;
+            }
+            s_issued = it;
+        }
+    } else if (warp == 9) {
+        if (lane == 0) {   // MMA issuer
+            const uint32_t idesc = tc_idesc(tile_n), w_lo = desc_lo(smem_u32(wsm), 16), ring_lo = desc_lo(smem_u32(smem), 16);
+            const int stage_lo = stage_bytes >> 4;
+            ok = weights = mbar_wait_try(smem_u32(wfull), 0u, TC_TIMEOUT_CYCLES);
+            int it = 0, st = 0, ph = 0, lt = 0;
+            for (int t = t0; t < t1 && ok;) {
+                const int is = t / s.h, ya = t - is * s.h, yb = min(s.h, ya + (t1 - t));
+                int p1 = 0, p2 = 0;   // the stages one and two rows back
+                for (int x = ya - 1; x <= yb; ++x) {
+                    if (!mbar_wait_try(smem_u32(&full[st]), ph, TC_TIMEOUT_CYCLES)) {
+                        ok = false;
+                        break;
+                    }
+                    if (x > ya) {   // the tile of row x - 1
+                        const int b = lt & 1;
+                        if (lt >= 2 && !mbar_wait_try(smem_u32(&acc_empty[b]), ((lt >> 1) - 1) & 1, TC_TIMEOUT_CYCLES)) {
+                            ok = false;
+                            ++it;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t d = tmem + (uint32_t)(b * tmem_cols);
+                        const uint32_t lo[3] = {ring_lo + (uint32_t)(p2 * stage_lo), ring_lo + (uint32_t)(p1 * stage_lo),
+                                                ring_lo + (uint32_t)(st * stage_lo)};
+                        uint32_t bl = w_lo;
+#pragma unroll
+                        for (int tap = 0; tap < 9; ++tap) {
+                            const int ddy = MODE == FWD ? tap / 3 - 1 : 1 - tap / 3, ddx = MODE == FWD ? tap % 3 - 1 : 1 - tap % 3;
+                            const uint32_t al = lo[ddy + 1] + (uint32_t)((1 + ddx) * rb / 16);
+#pragma unroll
+                            for (int ks = 0; ks < kc / 16; ++ks)
+                                tc_mma_lo(d, al + 2 * ks, desc_hi(rb), bl + 2 * ks, desc_hi(rb), idesc, (tap > 0 || ks > 0) ? 1u : 0u);
+                            bl += (uint32_t)(b_bytes >> 4);
+                        }
+                        tc_commit(smem_u32(&empty[p2]));
+                        if (x == yb) {
+                            tc_commit(smem_u32(&empty[p1]));
+                            tc_commit(smem_u32(&empty[st]));
+                        }
+                        tc_commit(smem_u32(&acc_full[b]));
+                        ++lt;
+                    }
+                    p2 = p1;
+                    p1 = st;
+                    ++it;
+                    if (++st == stages) {
+                        st = 0;
+                        ph ^= 1;
+                    }
+                }
+                t += yb - ya;
+            }
+            s_consumed = it;
+            tc_commit(smem_u32(done));   // arrives once every MMA issued above has completed
+        }
+    } else {   // epilogue: warps 0-3 the even tiles (accumulator 0), warps 4-7 the odd ones
+        const int quad = warp & 3;
+        const bool fast = !out_f32 && vec_out && tile_n % 32 == 0 && (sbias || !bias);
+        for (int lt = warp >> 2, t = t0 + lt; t < t1; t += 2, lt += 2) {
+            const int b = lt & 1;
+            const int is = t / s.h, y = t - is * s.h, img = is / segs, w0 = (is - img * segs) * TC_M;
+            const int row = (img * s.h + y) * s.w + w0 + quad * 32 + lane;
+            uint4 mk[4];
+            if (fast && mask) tm_mask_load(mask, row * N, mk);
+            if (!mbar_wait_try(smem_u32(&acc_full[b]), (lt >> 1) & 1, TC_TIMEOUT_CYCLES)) {
+                ok = false;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (fast)
+                tm_store_row32(tmem + (uint32_t)(b * tmem_cols) + ((uint32_t)(quad * 32) << 16), row * N, tile_n,
+                               sbias ? s_bias : nullptr, mask, mk, reinterpret_cast<__nv_bfloat16*>(out), relu);
+            else tm_store_row(tmem + (uint32_t)(b * tmem_cols) + ((uint32_t)(quad * 32) << 16), row, 0, N, tile_n, N,
+                         sbias ? s_bias : bias, mask, out, out_f32, relu, vec_out);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(smem_u32(&acc_empty[b]));
+        }
+    }
+    if (tid == 288) ok = mbar_wait_try(smem_u32(done), 0u, TC_TIMEOUT_CYCLES) && ok;
+    ok = __syncthreads_and(ok);
+    if (!ok && tid == 288) {
+        // loads still in flight write this CTA's shared memory: wait for them (bounded)
+        if (!weights) mbar_wait_try(smem_u32(wfull), 0u, TC_TIMEOUT_CYCLES);
+        for (int it = s_consumed; it < s_issued; ++it)
+            mbar_wait_try(smem_u32(&full[it % stages]), (it / stages) & 1, TC_TIMEOUT_CYCLES);
+        atomicExch(&g_nop_timeout, 1u);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 8)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * tmem_cols)
                      : "memory");
 }
@@ -1125,6 +1411,197 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tma(const __grid_constant_
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
 }
 
+// ---------------------------------------------------------------- row-ring weight gradient
+// Weight gradient of 3x3 layers whose channels come in atoms of 32, one image
+// row at a time: D[(tap, c)][n] = sum over pixels p of X[p + d(tap)][c] dY[p][n].
+// k_wgrad_tma fetches the activations once per tap (nine boxes per 64 pixels,
+// and each of its M tiles fetches dY again); its copies' request rate set the
+// pace.  Here a row of X, with one pixel of halo on either side, and the row of
+// dY below it are fetched once, into one stage of a ring; the three newest X
+// rows serve the taps dy = -1, 0, 1, and the taps dx = -1, 0, 1 are the same
+// bytes one pixel further on: both operands are MN-major (pixels along K), so
+// the M = 128 rows of an MMA are four 32-channel atoms whose leading byte
+// offset is one pixel (64 bytes; the swizzle follows the address).  The
+// fourth (dx = 2) is not stored.  Accumulators: a tile of tile_n columns per
+// (atom, dy), and with db one more whose A operand is a column of ones (its row
+// 0 is the bias gradient).  Rows are split over gridDim.z; gridDim.x takes
+// groups of `na` atoms, gridDim.y the output tiles.  16 x 128^2, 32 -> 32: 58.5
+// us before; see the launcher for the shapes.
+//   thread 0: copies, ring of `stages`; thread 32: MMAs; then warp j < 3 adds
+//   its rows (tap dx = j - 1) to dw with 16-byte reductions.
+// Every wait is bounded, as in k_conv_tma.
+constexpr int WR_ONES = 16 * 64;   // bytes of the ones operand: 16 K rows of 64 bytes
+
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+__global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant__ CUtensorMap mapX,
+                                                          const __grid_constant__ CUtensorMap mapY,
+                                                          float* __restrict__ dw, float* __restrict__ db, ConvShape s,
+                                                          int atoms, int na, int bw, int tile_n, int tmem_cols,
+                                                          int stages, int x_bytes, int y_bytes) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int atom0 = blockIdx.x * na, nc = min(na, atoms - atom0), n0 = blockIdx.y * tile_n;
+    const int nby = tile_n / bw;
+    const int stage_bytes = na * x_bytes + nby * y_bytes;          // both multiples of 1024
+    unsigned char* const ones = smem + stages * stage_bytes;       // 1024 bytes
+    uint64_t* full = reinterpret_cast<uint64_t*>(ones + WR_ONES);
+    uint64_t* empty = full + stages;
+    uint64_t* done = empty + stages;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    __shared__ int s_issued, s_consumed;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rows = s.n * s.h;
+    const int r0 = (int)((long long)rows * blockIdx.z / gridDim.z), r1 = (int)((long long)rows * (blockIdx.z + 1) / gridDim.z);
+    const bool bias = db && atom0 == 0;
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(smem_u32(&full[i]));
+            mbar_init(smem_u32(&empty[i]));
+        }
+        mbar_init(smem_u32(done));
+        s_issued = 0;
+        s_consumed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // the ones operand: channel 0 of every K row is 1, at its swizzled place
+    // (the 16-byte chunk of row k is XORed with k / 2 mod 4)
+    for (int i = tid; i < WR_ONES / 16; i += TC_THREADS) {
+        const int k = i >> 2, c = i & 3;
+        reinterpret_cast<uint4*>(ones)[i] = make_uint4(c == ((k >> 1) & 3) ? 0x3F80u : 0u, 0u, 0u, 0u);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+
+    // Both issuers walk the same items: for every run of rows [ya, yb) within
+    // an image, X rows ya - 1 .. yb, and with X row y + 1 the dY row y.
+    bool ok = true;
+    if (tid == 0) {   // copies
+        int it = 0, st = 0, ph = 0;
+        for (int r = r0; r < r1 && ok;) {
+            const int img = r / s.h, ya = r - img * s.h, yb = min(s.h, ya + (r1 - r));
+            for (int x = ya - 1; x <= yb; ++x) {
+                if (it >= stages && !mbar_wait_try(smem_u32(&empty[st]), ph ^ 1, TC_TIMEOUT_CYCLES)) {
+                    ok = false;
+                    break;
+                }
+                const int y = x - 1;
+                const uint32_t fb = smem_u32(&full[st]), base = smem_u32(smem + st * stage_bytes);
+                mbar_expect_tx(fb, (uint32_t)(nc * (s.w + 2) * 64 + (y >= ya ? nby * s.w * bw * 2 : 0)));
+                for (int j = 0; j < nc; ++j) tma_load_4d(base + j * x_bytes, &mapX, fb, (atom0 + j) * 32, -1, x, img);
+                if (y >= ya)
+                    for (int j = 0; j < nby; ++j)
+                        tma_load_4d(base + na * x_bytes + j * y_bytes, &mapY, fb, n0 + j * bw, 0, y, img);
+                ++it;
+                if (++st == stages) {
+                    st = 0;
+                    ph ^= 1;
+                }
+            }
+            r += yb - ya;
+        }
+        s_issued = it;
+    } else if (tid == 32) {   // MMAs
+        const uint32_t idesc = tc_idesc(tile_n) | (1u << 15) | (1u << 16);   // A and B MN-major
+        const uint32_t ring_lo = desc_lo(smem_u32(smem), 64), ones_lo = desc_lo(smem_u32(ones), 0);
+        const uint32_t by_lo = desc_lo(smem_u32(smem) + na * x_bytes, (uint32_t)y_bytes), bhi = desc_hi(2 * bw);
+        const int stage_lo = stage_bytes >> 4;
+        int it = 0, st = 0, ph = 0;
+        uint32_t acc = 0;
+        for (int r = r0; r < r1 && ok;) {
+            const int img = r / s.h, ya = r - img * s.h, yb = min(s.h, ya + (r1 - r));
+            int p1 = 0, p2 = 0;   // the stages one and two items back
+            for (int x = ya - 1; x <= yb; ++x) {
+                if (!mbar_wait_try(smem_u32(&full[st]), ph, TC_TIMEOUT_CYCLES)) {
+                    ok = false;
+                    break;
+                }
+                if (x > ya) {
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t lo[3] = {ring_lo + (uint32_t)(p2 * stage_lo), ring_lo + (uint32_t)(p1 * stage_lo),
+                                            ring_lo + (uint32_t)(st * stage_lo)};
+                    uint32_t bl = by_lo + (uint32_t)(st * stage_lo);
+                    for (int ks = 0; ks < s.w / 16; ++ks) {
+                        uint32_t d = tmem;
+                        for (int j = 0; j < nc; ++j) {
+                            const uint32_t off = (uint32_t)(j * (x_bytes >> 4) + ks * 64);
+#pragma unroll
+                            for (int dy = 0; dy < 3; ++dy) {
+                                tc_mma_lo(d, lo[dy] + off, desc_hi(64), bl, bhi, idesc, acc);
+                                d += (uint32_t)tile_n;
+                            }
+                        }
+                        if (bias) tc_mma_lo(tmem + (uint32_t)(3 * na * tile_n), ones_lo, desc_hi(64), bl, bhi, idesc, acc);
+                        bl += (uint32_t)(2 * bw);
+                        acc = 1;
+                    }
+                    tc_commit(smem_u32(&empty[p2]));
+                    if (x == yb) {   // the run's last rows are free too
+                        tc_commit(smem_u32(&empty[p1]));
+                        tc_commit(smem_u32(&empty[st]));
+                    }
+                }
+                p2 = p1;
+                p1 = st;
+                ++it;
+                if (++st == stages) {
+                    st = 0;
+                    ph ^= 1;
+                }
+            }
+            r += yb - ya;
+        }
+        s_consumed = it;
+        tc_commit(smem_u32(done));
+    }
+    ok = ok && mbar_wait_try(smem_u32(done), 0u, TC_TIMEOUT_CYCLES);
+    ok = __syncthreads_and(ok);
+    if (!ok && tid == 0) {
+        for (int it = s_consumed; it < s_issued; ++it)
+            mbar_wait_try(smem_u32(&full[it % stages]), (it / stages) & 1, TC_TIMEOUT_CYCLES);
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ok && r1 > r0) {
+        const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
+        for (int q = 0; q < 3 * nc + (bias ? 1 : 0); ++q) {
+            const bool is_bias = q == 3 * nc;
+            const int col = (is_bias ? 3 * na : q) * tile_n;
+            const int tap = (q % 3) * 3 + warp, c = (atom0 + q / 3) * 32 + lane;
+            float* dst = is_bias ? db + n0 : dw + (size_t)(tap * s.cin + c) * s.cout + n0;
+            const bool live = is_bias ? tid == 0 : warp < 3;
+            for (int c0 = 0; c0 < tile_n; c0 += 32) {
+                uint32_t v[32];
+                tc_ld32_nowait(lanes + (uint32_t)(col + c0), v);
+                tc_wait_ld();
+                if (live)
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        red_add4(dst + c0 + j, __uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]),
+                                 __uint_as_float(v[j + 3]));
+            }
+        }
+    } else if (!ok && tid == 0) {
+        atomicExch(&g_nop_timeout, 1u);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+}
+
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
 // Streaming multiprocessors of the current device (looked up once).
@@ -1235,8 +1712,8 @@ bool launch_tma(const void* A, const void* B, const float* bias, const void* mas
         if (!encode_map(&mb, B, 3, dims, strides, box, sw)) return false;
     }
     const size_t smem = 1024 + stages * stage_bytes + (2 * stages + 5) * 8 + 16;
-    if (cudaFuncSetAttribute(k_conv_tma<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess) {
+    const auto fn = kc == 64 ? k_conv_tma<MODE, 64> : k_conv_tma<MODE, 32>;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         *rc = CLB_NOP_ERR_CUDA;
         return true;
     }
@@ -1244,9 +1721,69 @@ bool launch_tma(const void* A, const void* B, const float* bias, const void* mas
     const long long ntiles = (M / TC_M) * ntn;
     const unsigned grid = (unsigned)std::min<long long>(ntiles, (long long)sm_count() * per_sm);
     const int vec_out = N % 8 == 0 && aligned16(out) && (!mask || aligned16(mask));
-    k_conv_tma<MODE><<<grid, TM_THREADS, smem, st>>>(ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu, s,
-                                                      (int)M, (int)N, tile_n, cols, vec_out, stages, cchunks, kc,
-                                                      (int)ntiles, ntn);
+    fn<<<grid, TM_THREADS, smem, st>>>(ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu, s, (int)M, (int)N,
+                                       tile_n, cols, vec_out, stages, cchunks, (int)ntiles, ntn);
+    *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
+    return true;
+}
+
+// Launches the row-ring kernel; false when the shape is not one it takes: 3x3,
+// width a multiple of 128, 32 input channels, at most 256 outputs (a multiple of
+// 16).  Measured at 16 x 128^2 against k_conv_tma (both with the present epilogue
+// and issue loops): 32 -> 32 20.9 us against 25.0, 32 -> 96 41 against 51; with
+// more input channels it is no faster (96 -> 32: 47.5 against 46.3) or slower
+// (3 x 128^2, 64 -> 64: 14.7 against 12.5: one CTA per SM), so those stay there.
+template <int MODE>
+bool launch_row(const void* A, const void* B, const float* bias, const void* mask, void* out, int out_f32, int relu,
+                ConvShape s, long long M, long long N, cudaStream_t st, int* rc) {
+    const int C = MODE == FWD ? s.cin : s.cout;
+    if (s.taps != 9 || s.w % TC_M || C != 32 || N % 16 || N > 256 || !aligned16(A) || !aligned16(B)) return false;
+    const long long cmax = s.cin > s.cout ? s.cin : s.cout;
+    if (M * cmax * s.taps >= 2147483647LL || M * N >= 2147483647LL) return false;
+    const int tile_n = (int)N;
+    int cols = 32;
+    while (cols < tile_n) cols <<= 1;
+    constexpr int kc = 32;
+    const int a_bytes = ((TC_M + 2) * kc * 2 + 1023) / 1024 * 1024;
+    const size_t w_bytes = (size_t)9 * tile_n * kc * 2, stage_bytes = (size_t)a_bytes;
+    // two CTAs per SM where TMEM and shared memory hold them (see launch_tma)
+    int per_sm = 2 * cols <= 256 ? 2 : 1;
+    long long stages = 0;
+    for (; per_sm >= 1; --per_sm) {
+        const long long budget = (per_sm == 2 ? 104 : 214) * 1024 - 1024 - 160 - (long long)w_bytes;
+        stages = std::min<long long>(CLB_ROW_MAX_STAGES, budget / (long long)stage_bytes);
+        if (stages >= 4) break;
+    }
+    if (stages < 4) return false;
+    CUtensorMap ma, mb;
+    const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_64B;
+    {
+        const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)s.w, (cuuint64_t)s.h, (cuuint64_t)s.n};
+        const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)s.w * C * 2, (cuuint64_t)s.h * s.w * C * 2};
+        const cuuint32_t box[4] = {(cuuint32_t)kc, TC_M + 2, 1, 1};
+        if (!encode_map(&ma, A, 4, dims, strides, box, sw)) return false;
+    }
+    if (MODE == FWD) {   // as launch_tma
+        const cuuint64_t dims[3] = {(cuuint64_t)s.cin, (cuuint64_t)s.taps, (cuuint64_t)s.cout};
+        const cuuint64_t strides[2] = {(cuuint64_t)s.cin * 2, (cuuint64_t)s.taps * s.cin * 2};
+        const cuuint32_t box[3] = {(cuuint32_t)kc, 1, (cuuint32_t)tile_n};
+        if (!encode_map(&mb, B, 3, dims, strides, box, sw)) return false;
+    } else {
+        const cuuint64_t dims[3] = {(cuuint64_t)s.cout, (cuuint64_t)s.cin, (cuuint64_t)s.taps};
+        const cuuint64_t strides[2] = {(cuuint64_t)s.cout * 2, (cuuint64_t)s.cin * s.cout * 2};
+        const cuuint32_t box[3] = {(cuuint32_t)kc, (cuuint32_t)tile_n, 1};
+        if (!encode_map(&mb, B, 3, dims, strides, box, sw)) return false;
+    }
+    const size_t smem = 1024 + w_bytes + stages * stage_bytes + (2 * stages + 6) * 8 + 16;
+    if (cudaFuncSetAttribute(k_conv_row<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        *rc = CLB_NOP_ERR_CUDA;
+        return true;
+    }
+    const long long total = M / TC_M;
+    const unsigned grid = (unsigned)std::min<long long>(total, (long long)sm_count() * per_sm);
+    const int vec_out = N % 8 == 0 && aligned16(out) && (!mask || aligned16(mask));
+    k_conv_row<MODE><<<grid, TM_THREADS, smem, st>>>(ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu, s, (int)N,
+                                                     tile_n, cols, vec_out, (int)stages, a_bytes, (int)total);
     *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     return true;
 }
@@ -1351,6 +1888,56 @@ bool launch_wgrad_tma(const void* x, const void* dy, float* dw, float* db, ConvS
                                                 ones_atom);
     *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     *bias_done = ones_atom >= 0;
+    return true;
+}
+
+// Launches the row-ring weight gradient; false when the shape is not one it
+// takes: 3x3, channels in multiples of 32, rows of a multiple of 16 pixels that
+// fit a copy box with their halo.  db is always filled.
+bool launch_wgrad_row(const void* x, const void* dy, float* dw, float* db, ConvShape s, int splitk, cudaStream_t st,
+                      int* rc) {
+    if (s.taps != 9 || s.cin % 32 || s.cout % 32 || s.w % 16 || s.w > 240) return false;
+    if (!aligned16(x) || !aligned16(dy) || !aligned16(dw) || (db && !aligned16(db))) return false;
+    const long long npix = (long long)s.n * s.h * s.w;
+    if (npix * (s.cin > s.cout ? s.cin : s.cout) * s.taps >= 2147483647LL) return false;
+    // output tile: the whole of narrow layers, else 64 or 32 columns; then as
+    // many atoms as their three accumulators and the bias's fit in TMEM
+    const int tile_n = s.cout <= 96 ? s.cout : s.cout % 64 == 0 ? 64 : 32;
+    const int bw = tile_n % 64 == 0 ? 64 : 32;
+    const int atoms = s.cin / 32, na = std::min(atoms, (512 / tile_n - 1) / 3);
+    const int groups = (atoms + na - 1) / na, ntn = s.cout / tile_n;
+    int cols = 32;
+    while (cols < (3 * na + 1) * tile_n) cols <<= 1;
+    const int x_bytes = ((s.w + 3) * 64 + 1023) / 1024 * 1024, y_bytes = (s.w * bw * 2 + 1023) / 1024 * 1024;
+    const size_t stage_bytes = (size_t)na * x_bytes + (size_t)(tile_n / bw) * y_bytes;
+    const int stages = (int)std::min<size_t>(CLB_WR_MAX_STAGES, (200 * 1024) / stage_bytes);
+    if (stages < 4) return false;
+    const int rows = s.n * s.h;
+    long long gz = splitk >= 1 ? splitk : std::max(1, CLB_WR_CTAS * sm_count() / (groups * ntn));
+    gz = std::max(1LL, std::min(gz, splitk >= 1 ? (long long)rows : (long long)(rows + 3) / 4));
+    if (gz > 65535) return false;
+    CUtensorMap mx, my;
+    {
+        const cuuint64_t dims[4] = {(cuuint64_t)s.cin, (cuuint64_t)s.w, (cuuint64_t)s.h, (cuuint64_t)s.n};
+        const cuuint64_t strides[3] = {(cuuint64_t)s.cin * 2, (cuuint64_t)s.w * s.cin * 2, (cuuint64_t)s.h * s.w * s.cin * 2};
+        const cuuint32_t box[4] = {32, (cuuint32_t)(s.w + 2), 1, 1};
+        if (!encode_map(&mx, x, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B)) return false;
+    }
+    {
+        const cuuint64_t dims[4] = {(cuuint64_t)s.cout, (cuuint64_t)s.w, (cuuint64_t)s.h, (cuuint64_t)s.n};
+        const cuuint64_t strides[3] = {(cuuint64_t)s.cout * 2, (cuuint64_t)s.w * s.cout * 2, (cuuint64_t)s.h * s.w * s.cout * 2};
+        const cuuint32_t box[4] = {(cuuint32_t)bw, (cuuint32_t)s.w, 1, 1};
+        if (!encode_map(&my, dy, 4, dims, strides, box, bw == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
+            return false;
+    }
+    const size_t smem = 1024 + stages * stage_bytes + WR_ONES + (2 * stages + 1) * 8 + 16;
+    if (cudaFuncSetAttribute(k_wgrad_row, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        *rc = CLB_NOP_ERR_CUDA;
+        return true;
+    }
+    k_wgrad_row<<<dim3((unsigned)groups, (unsigned)ntn, (unsigned)gz), TC_THREADS, smem, st>>>(
+        mx, my, dw, db, s, atoms, na, bw, tile_n, cols, stages, x_bytes, y_bytes);
+    *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     return true;
 }
 
@@ -1822,6 +2409,8 @@ extern "C" int clb_nop_conv_fwd(const void* x, const void* w, const void* wt, co
     const ConvShape s{n, h, wd, cin, cout, taps};
     const long long M = (long long)n * h * wd, K = (long long)taps * cin;
     int rc;
+    if (wt && launch_row<FWD>(x, wt, bias, nullptr, y, y_f32, relu, s, M, cout, (cudaStream_t)stream, &rc))
+        return rc;
     if (wt && launch_tma<FWD>(x, wt, bias, nullptr, y, y_f32, relu, s, M, cout, (cudaStream_t)stream, &rc))
         return rc;
     if (wt && launch_tc<FWD>(x, wt, bias, nullptr, y, y_f32, relu, s, M, cout, K, (cudaStream_t)stream, &rc))
@@ -1835,6 +2424,7 @@ extern "C" int clb_nop_conv_dgrad(const void* dy, const void* w, const void* mas
     const ConvShape s{n, h, wd, cin, cout, taps};
     const long long M = (long long)n * h * wd, K = (long long)taps * cout;
     int rc;
+    if (launch_row<DGRAD>(dy, w, nullptr, mask, dx, 0, 0, s, M, cin, (cudaStream_t)stream, &rc)) return rc;
     if (launch_tma<DGRAD>(dy, w, nullptr, mask, dx, 0, 0, s, M, cin, (cudaStream_t)stream, &rc)) return rc;
     if (launch_tc<DGRAD>(dy, w, nullptr, mask, dx, 0, 0, s, M, cin, K, (cudaStream_t)stream, &rc)) return rc;
     if (launch_dgrad_small(dy, w, mask, dx, s, (cudaStream_t)stream, &rc)) return rc;
@@ -1849,6 +2439,7 @@ extern "C" int clb_nop_conv_wgrad_bias(const void* x, const void* dy, float* dw,
     const cudaStream_t st = (cudaStream_t)stream;
     int rc;
     bool bias_done = false;
+    if (launch_wgrad_row(x, dy, dw, db, s, splitk, st, &rc)) return rc;
     if (launch_wgrad_tma(x, dy, dw, db, s, splitk, st, &rc, &bias_done)) {
         if (rc != CLB_NOP_OK || !db || bias_done) return rc;
         return clb_nop_bias_grad(dy, db, (int64_t)n * h * wd, cout, stream);
