@@ -135,6 +135,41 @@ int clb_nop_check(void* stream);
  * detection. */
 int clb_nop_wait_selftest(int64_t limit_cycles, void* stream);
 
+/* One convolution of the warm-start network: BF16 weights [taps * cin][cout]
+ * and their transpose, FP32 bias, ReLU or not. */
+typedef struct {
+    const void* w;
+    const void* wt;
+    const float* bias;
+    int32_t cin, cout, taps, relu;
+} clb_nop_layer;
+
+/* The warm-start network's forward pass in one call: 15 layers (encoder 0-5,
+ * bottom 6-7, decoder 8-13, head 14; each decoder level starts with [nearest 2x
+ * upsampling | skip]) on n images of h x w, multiples of 8.
+ * clb_nop_net_acts: bytes of all activations, 0 if the layers do not fit
+ * together; offsets (21, or NULL) receives where each starts: padded input,
+ * a1, a2, pool1, a3, a4, pool2, a5, a6, pool3, a7, a8, cat3, a9, a10, cat2, a11,
+ * a12, cat1, a13, a14.
+ * clb_nop_net_forward: x is BF16 (n, h, w, n_in), padded with zeros to
+ * layer 0's channels; acts holds clb_nop_net_acts bytes (16-byte aligned), out is
+ * FP32 (n, h, w, cout of layer 14).  The same kernels as the calls above, so the
+ * same values. */
+int64_t clb_nop_net_acts(const clb_nop_layer* layers, int32_t n, int32_t h, int32_t w, int64_t* offsets);
+int clb_nop_net_forward(const clb_nop_layer* layers, const void* x, int32_t n_in, void* acts, float* out, int32_t n,
+                        int32_t h, int32_t w, void* stream);
+
+/* The backward pass in one call: acts are the 21 activations of the forward
+ * pass (in the order of clb_nop_net_acts), dout the BF16 gradient of the output;
+ * adds every layer's weight and bias gradient to gw[l] and gb[l] (FP32; clear
+ * them first).  The weight gradients run on side_stream beside the
+ * input-gradient chain; stream waits for them at the end.  scratch:
+ * clb_nop_net_scratch bytes, 16-byte aligned, in use until stream gets there. */
+int64_t clb_nop_net_scratch(const clb_nop_layer* layers, int32_t n, int32_t h, int32_t w);
+int clb_nop_net_backward(const clb_nop_layer* layers, float* const* gw, float* const* gb, const void* const* acts,
+                         const void* dout, void* scratch, int32_t n, int32_t h, int32_t w, void* stream,
+                         void* side_stream);
+
 /* Clear `bytes` bytes at ptr. */
 int clb_nop_zero(void* ptr, int64_t bytes, void* stream);
 

@@ -34,6 +34,26 @@
 
 namespace {
 
+// Programmatic dependent launch, for the kernels of a forward pass: their
+// blocks may start (and set up barriers, TMEM, tensor maps) before the kernel
+// in front of them has ended, and wait here before they touch its results.
+__device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... V>
+void launch_pdl(void (*k)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, const V&... v) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, P(v)...);   // an error stays for the caller's cudaGetLastError
+}
+
 constexpr int BM = 64, BN = 64, BK = 32, PAD = 8;
 constexpr int kThreads = 128;
 
@@ -770,6 +790,10 @@ __global__ void __launch_bounds__(TM_THREADS, 2) k_conv_tma(const __grid_constan
         s_consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // every CTA holds its TMEM before the next kernel's may ask for theirs
+    __syncthreads();
+    pdl_start();
+    pdl_wait();
     const bool sbias = bias && N <= TM_BIAS_MAX;
     if (sbias)
         for (int i = tid; i < N; i += TM_THREADS) s_bias[i] = bias[i];
@@ -938,6 +962,10 @@ __global__ void __launch_bounds__(TM_THREADS, 2)
         s_consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // every CTA holds its TMEM before the next kernel's may ask for theirs
+    __syncthreads();
+    pdl_start();
+    pdl_wait();
     const bool sbias = bias && N <= TM_BIAS_MAX;
     if (sbias)
         for (int i = tid; i < N; i += TM_THREADS) s_bias[i] = bias[i];
@@ -1721,8 +1749,8 @@ bool launch_tma(const void* A, const void* B, const float* bias, const void* mas
     const long long ntiles = (M / TC_M) * ntn;
     const unsigned grid = (unsigned)std::min<long long>(ntiles, (long long)sm_count() * per_sm);
     const int vec_out = N % 8 == 0 && aligned16(out) && (!mask || aligned16(mask));
-    fn<<<grid, TM_THREADS, smem, st>>>(ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu, s, (int)M, (int)N,
-                                       tile_n, cols, vec_out, stages, cchunks, (int)ntiles, ntn);
+    launch_pdl(fn, dim3(grid), TM_THREADS, smem, st, ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu, s, (int)M,
+               (int)N, tile_n, cols, vec_out, stages, cchunks, (int)ntiles, ntn);
     *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     return true;
 }
@@ -1782,8 +1810,8 @@ bool launch_row(const void* A, const void* B, const float* bias, const void* mas
     const long long total = M / TC_M;
     const unsigned grid = (unsigned)std::min<long long>(total, (long long)sm_count() * per_sm);
     const int vec_out = N % 8 == 0 && aligned16(out) && (!mask || aligned16(mask));
-    k_conv_row<MODE><<<grid, TM_THREADS, smem, st>>>(ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu, s, (int)N,
-                                                     tile_n, cols, vec_out, (int)stages, a_bytes, (int)total);
+    launch_pdl(k_conv_row<MODE>, dim3(grid), TM_THREADS, smem, st, ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu,
+               s, (int)N, tile_n, cols, vec_out, (int)stages, a_bytes, (int)total);
     *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     return true;
 }
@@ -2130,7 +2158,9 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
 }
 
 // n * h * w pixels of G = c / 8 vectors; vector index i -> (pixel, group)
-__global__ void k_pool2_fwd8(const uint4* __restrict__ x, uint4* __restrict__ y, int n, int h, int w, int G) {
+__global__ void k_pool2_fwd8(const uint4* x, uint4* __restrict__ y, int n, int h, int w, int G) {
+    pdl_start();
+    pdl_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int ho = h / 2, wo = w / 2;
     if (i >= (long long)n * ho * wo * G) return;
@@ -2220,6 +2250,101 @@ __global__ void k_concat8(uint4* __restrict__ a, uint4* __restrict__ b, uint4* _
     uint4* src = g < ga ? a + p * ga + g : b + p * gb + (g - ga);
     if (!inverse) y[i] = *src;
     else *src = y[i];
+}
+
+// y (n, 2h, 2w, ca + cb) = [nearest 2x upsampling of a (n, h, w, ca) | b (n, 2h,
+// 2w, cb)]: the decoder's skip connection without the upsampled copy.
+__global__ void k_upcat8(const uint4* a, const uint4* b, uint4* __restrict__ y, int n, int h, int w, int ga, int gb) {
+    pdl_start();
+    pdl_wait();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int H = 2 * h, W = 2 * w, G = ga + gb;
+    if (i >= (long long)n * H * W * G) return;
+    const long long p = i / G;
+    const int g = (int)(i - p * G);
+    if (g >= ga) {
+        y[i] = b[p * gb + (g - ga)];
+        return;
+    }
+    const long long q = p / W;
+    const int X = (int)(p - q * W), bi = (int)(q / H), Y = (int)(q - (long long)bi * H);
+    y[i] = a[(((long long)bi * h + Y / 2) * w + X / 2) * ga + g];
+}
+
+// Backward of the skip connection's upsampled part: dy (n, 2h, 2w, gs vectors)
+// holds the gradient of [up(a) | skip]; dx (n, h, w, ga) = sum of the four
+// copies of a's part, zeroed where a <= 0.  Rounded to BF16 before the mask as
+// the separate passes (split, upsampling backward, mask) did: the same bits.
+__global__ void k_up2_bwd_mask8(const uint4* dy, const uint4* __restrict__ a, uint4* __restrict__ dx, int n, int h, int w,
+                                int ga, int gs) {
+    pdl_start();
+    pdl_wait();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (long long)n * h * w * ga) return;
+    const long long p = i / ga;
+    const int g = (int)(i - p * ga);
+    const long long q = p / w;
+    const int x = (int)(p - q * w);   // q = image * h + row: the upper left copy is at row 2 q
+    const long long base = (4 * q * w + 2 * x) * gs + g, row = 2LL * w * gs;
+    float s[8], t[8];
+    unpack8(dy[base], s);
+    unpack8(dy[base + gs], t);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] += t[j];
+    unpack8(dy[base + row], t);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] += t[j];
+    unpack8(dy[base + row + gs], t);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] += t[j];
+    unpack8(a[i], t);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (!(t[j] > 0.0f)) s[j] = 0.0f;
+    dx[i] = pack8(s);
+}
+
+// Gradient of an encoder output a (n, h, w, G vectors) that goes both into the
+// 2x2 pooling (dp: its gradient, (n, h/2, w/2, G)) and into a skip connection
+// (ds: gradient of [up | a], gs vectors per pixel, a's part from vector go):
+// dp / 4 (rounded to BF16, as the pooling's own backward pass gives it) + ds's
+// part, zeroed where a <= 0.
+__global__ void k_pool2_bwd_skip8(const uint4* dp, const uint4* ds, const uint4* __restrict__ a, uint4* __restrict__ dx, int n,
+                                  int h, int w, int G, int gs, int go) {
+    pdl_start();
+    pdl_wait();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (long long)n * h * w * G) return;
+    const long long p = i / G;
+    const int g = (int)(i - p * G);
+    const long long q = p / w;
+    const int x = (int)(p - q * w), b = (int)(q / h), y = (int)(q - (long long)b * h);
+    float s[8], t[8];
+    unpack8(dp[(((long long)b * (h / 2) + y / 2) * (w / 2) + x / 2) * G + g], s);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] *= 0.25f;
+    unpack8(pack8(s), s);
+    unpack8(ds[p * gs + go + g], t);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] += t[j];
+    unpack8(a[i], t);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (!(t[j] > 0.0f)) s[j] = 0.0f;
+    dx[i] = pack8(s);
+}
+
+// y (npix, gx + gz) = [x | zeros], T: a 16-byte vector or one value.
+template <typename T>
+__global__ void k_pad(const T* x, T* __restrict__ y, long long npix, int gx, int gz) {
+    pdl_start();
+    pdl_wait();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int G = gx + gz;
+    if (i >= npix * G) return;
+    const long long p = i / G;
+    const int g = (int)(i - p * G);
+    y[i] = g < gx ? x[p * gx + g] : T{};
 }
 
 __global__ void k_add_mask8(const uint4* __restrict__ d1, const uint4* __restrict__ d2, const uint4* __restrict__ a,
@@ -2335,6 +2460,8 @@ __global__ void __launch_bounds__(256) k_dgrad_small(const __nv_bfloat16* __rest
                                                      const __nv_bfloat16* __restrict__ mask,
                                                      __nv_bfloat16* __restrict__ dx, long long npix) {
     __shared__ float sw[CIN * COUT];
+    pdl_start();
+    pdl_wait();
     for (int k = threadIdx.x; k < CIN * COUT; k += blockDim.x) sw[k] = __bfloat162float(w[k]);
     __syncthreads();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2372,10 +2499,10 @@ bool launch_dgrad_small(const void* dy, const void* w, const void* mask, void* d
     const __nv_bfloat16 *dyb = (const __nv_bfloat16*)dy, *wb = (const __nv_bfloat16*)w,
                         *mb = (const __nv_bfloat16*)mask;
     __nv_bfloat16* dxb = (__nv_bfloat16*)dx;
-    if (s.cout == 4 && s.cin == 8) k_dgrad_small<8, 4><<<grid, 256, 0, st>>>(dyb, wb, mb, dxb, npix);
-    else if (s.cout == 4 && s.cin == 16) k_dgrad_small<16, 4><<<grid, 256, 0, st>>>(dyb, wb, mb, dxb, npix);
-    else if (s.cout == 4 && s.cin == 24) k_dgrad_small<24, 4><<<grid, 256, 0, st>>>(dyb, wb, mb, dxb, npix);
-    else if (s.cout == 4 && s.cin == 32) k_dgrad_small<32, 4><<<grid, 256, 0, st>>>(dyb, wb, mb, dxb, npix);
+    if (s.cout == 4 && s.cin == 8) launch_pdl(k_dgrad_small<8, 4>, dim3(grid), 256, 0, st, dyb, wb, mb, dxb, npix);
+    else if (s.cout == 4 && s.cin == 16) launch_pdl(k_dgrad_small<16, 4>, dim3(grid), 256, 0, st, dyb, wb, mb, dxb, npix);
+    else if (s.cout == 4 && s.cin == 24) launch_pdl(k_dgrad_small<24, 4>, dim3(grid), 256, 0, st, dyb, wb, mb, dxb, npix);
+    else if (s.cout == 4 && s.cin == 32) launch_pdl(k_dgrad_small<32, 4>, dim3(grid), 256, 0, st, dyb, wb, mb, dxb, npix);
     else return false;
     *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     return true;
@@ -2478,8 +2605,8 @@ extern "C" int clb_nop_pool2(const void* in, void* out, int32_t n, int32_t h, in
     if (c % 8 == 0 && aligned16(in) && aligned16(out)) {
         const int G = c / 8;
         if (!backward)
-            k_pool2_fwd8<<<nblk((long long)n * (h / 2) * (w / 2) * G), 256, 0, st>>>((const uint4*)in, (uint4*)out, n, h,
-                                                                                    w, G);
+            launch_pdl(k_pool2_fwd8, dim3(nblk((long long)n * (h / 2) * (w / 2) * G)), 256, 0, st, (const uint4*)in, (uint4*)out,
+                       n, h, w, G);
         else
             k_pool2_bwd8<<<nblk((long long)n * h * w * G), 256, 0, st>>>((const uint4*)in, (uint4*)out, n, h, w, G);
         return status();
@@ -2708,4 +2835,198 @@ extern "C" int clb_nop_check(void* stream) {
     if (cudaMemcpyFromSymbol(&flag, g_nop_timeout, sizeof(flag)) != cudaSuccess) return CLB_NOP_ERR_CUDA;
     if (flag && cudaMemcpyToSymbol(g_nop_timeout, &zero, sizeof(zero)) != cudaSuccess) return CLB_NOP_ERR_CUDA;
     return flag ? CLB_NOP_ERR_TIMEOUT : CLB_NOP_OK;
+}
+
+// ---------------------------------------------------------------- forward pass
+// Activation slots of the network's forward pass, in the order of
+// clb_nop_net_acts; a slot starts on a 256-byte boundary.
+namespace {
+constexpr int kNetLayers = 15, kNetActs = 21;
+enum { AX, A1, A2, AP1, A3, A4, AP2, A5, A6, AP3, A7, A8, AC3, A9, A10, AC2, A11, A12, AC1, A13, A14 };
+
+// Bytes of the activations of n images of h x w, and each one's offset; 0 if
+// the layers do not fit together or the sizes are not multiples of 8 pixels.
+int64_t net_layout(const clb_nop_layer* L, int n, int h, int w, int64_t* off) {
+    if (n < 1 || h < 8 || w < 8 || h % 8 || w % 8) return 0;
+    for (int i = 0; i < kNetLayers; ++i)
+        if (!L[i].w || L[i].cin < 1 || L[i].cout < 1 || L[i].taps != (i < 14 ? 9 : 1) || (i < 14 && (L[i].cin % 8 || L[i].cout % 8)))
+            return 0;
+    const int chain[14] = {L[0].cin, L[0].cout, L[1].cout, L[2].cout, L[3].cout, L[4].cout, L[5].cout,
+                           L[6].cout, L[7].cout + L[5].cout, L[8].cout, L[9].cout + L[3].cout, L[10].cout,
+                           L[11].cout + L[1].cout, L[12].cout};   // inputs of layers 0 .. 13
+    for (int i = 0; i < 14; ++i)
+        if (L[i].cin != chain[i]) return 0;
+    if (L[14].cin != L[13].cout) return 0;
+    const int c[kNetActs] = {L[0].cin,  L[0].cout, L[1].cout, L[1].cout, L[2].cout,  L[3].cout,  L[3].cout,
+                             L[4].cout, L[5].cout, L[5].cout, L[6].cout, L[7].cout,  L[8].cin,   L[8].cout,
+                             L[9].cout, L[10].cin, L[10].cout, L[11].cout, L[12].cin, L[12].cout, L[13].cout};
+    const int d[kNetActs] = {1, 1, 1, 2, 2, 2, 4, 4, 4, 8, 8, 8, 4, 4, 4, 2, 2, 2, 1, 1, 1};
+    int64_t at = 0;
+    for (int i = 0; i < kNetActs; ++i) {
+        if (off) off[i] = at;
+        at += ((int64_t)n * (h / d[i]) * (w / d[i]) * c[i] * 2 + 255) / 256 * 256;
+    }
+    return at;
+}
+}  // namespace
+
+extern "C" int64_t clb_nop_net_acts(const clb_nop_layer* layers, int32_t n, int32_t h, int32_t w, int64_t* offsets) {
+    return layers ? net_layout(layers, n, h, w, offsets) : 0;
+}
+
+extern "C" int clb_nop_net_forward(const clb_nop_layer* L, const void* x, int32_t n_in, void* acts, float* out, int32_t n,
+                                   int32_t h, int32_t w, void* stream) {
+    if (!L || !x || !acts || !out || !aligned16(acts)) return CLB_NOP_ERR_ARG;
+    int64_t off[kNetActs];
+    if (!net_layout(L, n, h, w, off) || n_in < 1 || n_in > L[0].cin) return CLB_NOP_ERR_ARG;
+    const cudaStream_t st = (cudaStream_t)stream;
+    auto at = [&](int i) { return (char*)acts + off[i]; };
+    int rc = CLB_NOP_OK;
+    auto conv = [&](int l, int in, void* y, int d) {
+        if (rc == CLB_NOP_OK)
+            rc = clb_nop_conv_fwd(at(in), L[l].w, L[l].wt, L[l].bias, y, l == 14, L[l].relu, n, h / d, w / d, L[l].cin, L[l].cout,
+                                  L[l].taps, stream);
+    };
+    auto pool = [&](int in, int y, int d, int c) {
+        if (rc == CLB_NOP_OK) rc = clb_nop_pool2(at(in), at(y), n, h / d, w / d, c, 0, stream);
+    };
+    auto upcat = [&](int a, int b, int y, int d, int ca, int cb) {   // a at 1/d of the resolution, b and y at 2/d
+        if (rc != CLB_NOP_OK) return;
+        const long long n8 = 4LL * n * (h / d) * (w / d) * ((ca + cb) / 8);
+        launch_pdl(k_upcat8, dim3(nblk(n8)), 256, 0, st, (const uint4*)at(a), (const uint4*)at(b), (uint4*)at(y), n, h / d, w / d,
+                   ca / 8, cb / 8);
+        rc = status();
+    };
+    const long long npix = (long long)n * h * w;
+    if (n_in % 8 == 0 && aligned16(x))
+        launch_pdl(k_pad<uint4>, dim3(nblk(npix * (L[0].cin / 8))), 256, 0, st, (const uint4*)x, (uint4*)at(AX), npix, n_in / 8,
+                   (L[0].cin - n_in) / 8);
+    else
+        launch_pdl(k_pad<uint16_t>, dim3(nblk(npix * L[0].cin)), 256, 0, st, (const uint16_t*)x, (uint16_t*)at(AX), npix, n_in,
+                   L[0].cin - n_in);
+    rc = status();
+    conv(0, AX, at(A1), 1);
+    conv(1, A1, at(A2), 1);
+    pool(A2, AP1, 1, L[1].cout);
+    conv(2, AP1, at(A3), 2);
+    conv(3, A3, at(A4), 2);
+    pool(A4, AP2, 2, L[3].cout);
+    conv(4, AP2, at(A5), 4);
+    conv(5, A5, at(A6), 4);
+    pool(A6, AP3, 4, L[5].cout);
+    conv(6, AP3, at(A7), 8);
+    conv(7, A7, at(A8), 8);
+    upcat(A8, A6, AC3, 8, L[7].cout, L[5].cout);
+    conv(8, AC3, at(A9), 4);
+    conv(9, A9, at(A10), 4);
+    upcat(A10, A4, AC2, 4, L[9].cout, L[3].cout);
+    conv(10, AC2, at(A11), 2);
+    conv(11, A11, at(A12), 2);
+    upcat(A12, A2, AC1, 2, L[11].cout, L[1].cout);
+    conv(12, AC1, at(A13), 1);
+    conv(13, A13, at(A14), 1);
+    conv(14, A14, out, 1);
+    return rc;
+}
+
+// ---------------------------------------------------------------- backward pass
+namespace {
+// Gradient buffers of the backward pass: dx of layers 14 .. 1 (input gradients,
+// masked where their input is a layer's output) and the six joins.
+constexpr int kNetGrads = 14 + 6;
+int64_t net_grad_layout(const clb_nop_layer* L, int n, int h, int w, int64_t* off) {
+    if (!net_layout(L, n, h, w, nullptr)) return 0;
+    const int res[kNetLayers] = {1, 1, 2, 2, 4, 4, 8, 8, 4, 4, 2, 2, 1, 1, 1};
+    int64_t at = 0;
+    auto take = [&](int i, int d, int c) {
+        if (off) off[i] = at;
+        at += ((int64_t)n * (h / d) * (w / d) * c * 2 + 255) / 256 * 256;
+    };
+    for (int l = 1; l <= 14; ++l) take(l - 1, res[l], L[l].cin);   // slot l - 1: dx of layer l
+    take(14, 2, L[11].cout);   // d a12
+    take(15, 4, L[9].cout);    // d a10
+    take(16, 8, L[7].cout);    // d a8
+    take(17, 4, L[5].cout);    // d a6
+    take(18, 2, L[3].cout);    // d a4
+    take(19, 1, L[1].cout);    // d a2
+    return at;
+}
+}  // namespace
+
+extern "C" int64_t clb_nop_net_scratch(const clb_nop_layer* layers, int32_t n, int32_t h, int32_t w) {
+    return layers ? net_grad_layout(layers, n, h, w, nullptr) : 0;
+}
+
+extern "C" int clb_nop_net_backward(const clb_nop_layer* L, float* const* gw, float* const* gb, const void* const* acts,
+                                    const void* dout, void* scratch, int32_t n, int32_t h, int32_t w, void* stream,
+                                    void* side_stream) {
+    if (!L || !gw || !gb || !acts || !dout || !scratch || !aligned16(scratch)) return CLB_NOP_ERR_ARG;
+    int64_t off[kNetGrads];
+    if (!net_grad_layout(L, n, h, w, off)) return CLB_NOP_ERR_ARG;
+    for (int i = 0; i < kNetActs; ++i)
+        if (!acts[i] || !aligned16(acts[i])) return CLB_NOP_ERR_ARG;
+    for (int i = 0; i < kNetLayers; ++i)
+        if (!gw[i] || !gb[i]) return CLB_NOP_ERR_ARG;
+    const cudaStream_t st = (cudaStream_t)stream, side = (cudaStream_t)side_stream;
+    cudaEvent_t ev = nullptr;
+    if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) return CLB_NOP_ERR_CUDA;
+    auto G = [&](int i) -> void* { return (char*)scratch + off[i]; };
+    const int res[kNetLayers] = {1, 1, 2, 2, 4, 4, 8, 8, 4, 4, 2, 2, 1, 1, 1};
+    int rc = CLB_NOP_OK;
+    // Layer l: weight and bias gradient on the side stream (nothing before the
+    // optimiser needs them), then the input gradient on the main one.
+    auto layer = [&](int l, int in, const void* dy, bool masked) {
+        if (rc != CLB_NOP_OK) return;
+        const int hh = h / res[l], ww = w / res[l];
+        if (cudaEventRecord(ev, st) != cudaSuccess || cudaStreamWaitEvent(side, ev, 0) != cudaSuccess) {
+            rc = CLB_NOP_ERR_CUDA;
+            return;
+        }
+        rc = clb_nop_conv_wgrad_bias(acts[in], dy, gw[l], gb[l], n, hh, ww, L[l].cin, L[l].cout, L[l].taps, 0, side_stream);
+        if (rc == CLB_NOP_OK && l > 0)
+            rc = clb_nop_conv_dgrad(dy, L[l].w, masked ? acts[in] : nullptr, G(l - 1), n, hh, ww, L[l].cin, L[l].cout, L[l].taps,
+                                    stream);
+    };
+    // d a (at 1/d of the resolution) from the gradient of [up(a) | skip] at 2/d
+    auto up = [&](const void* dc, int act, int slot, int d, int ca, int cb) {
+        if (rc != CLB_NOP_OK) return;
+        const long long n8 = (long long)n * (h / d) * (w / d) * (ca / 8);
+        launch_pdl(k_up2_bwd_mask8, dim3(nblk(n8)), 256, 0, st, (const uint4*)dc, (const uint4*)acts[act], (uint4*)G(slot), n, h / d,
+                   w / d, ca / 8, (ca + cb) / 8);
+        rc = status();
+    };
+    // d a of an encoder output (at 1/d) from its pooling's and its skip's gradients
+    auto join = [&](const void* dp, const void* dc, int act, int slot, int d, int ca, int cb) {
+        if (rc != CLB_NOP_OK) return;
+        const long long n8 = (long long)n * (h / d) * (w / d) * (cb / 8);
+        launch_pdl(k_pool2_bwd_skip8, dim3(nblk(n8)), 256, 0, st, (const uint4*)dp, (const uint4*)dc, (const uint4*)acts[act],
+                   (uint4*)G(slot), n, h / d, w / d, cb / 8, (ca + cb) / 8, ca / 8);
+        rc = status();
+    };
+    layer(14, A14, dout, true);
+    layer(13, A13, G(13), true);
+    layer(12, AC1, G(12), false);
+    up(G(11), A12, 14, 2, L[11].cout, L[1].cout);
+    layer(11, A11, G(14), true);
+    layer(10, AC2, G(10), false);
+    up(G(9), A10, 15, 4, L[9].cout, L[3].cout);
+    layer(9, A9, G(15), true);
+    layer(8, AC3, G(8), false);
+    up(G(7), A8, 16, 8, L[7].cout, L[5].cout);
+    layer(7, A7, G(16), true);
+    layer(6, AP3, G(6), false);
+    join(G(5), G(7), A6, 17, 4, L[7].cout, L[5].cout);
+    layer(5, A5, G(17), true);
+    layer(4, AP2, G(4), false);
+    join(G(3), G(9), A4, 18, 2, L[9].cout, L[3].cout);
+    layer(3, A3, G(18), true);
+    layer(2, AP1, G(2), false);
+    join(G(1), G(11), A2, 19, 1, L[11].cout, L[1].cout);
+    layer(1, A1, G(19), true);
+    layer(0, AX, G(0), false);
+    // whatever runs next on the main stream finds every gradient (also after an error: nothing may still read the buffers)
+    if (cudaEventRecord(ev, side) != cudaSuccess || cudaStreamWaitEvent(st, ev, 0) != cudaSuccess)
+        if (rc == CLB_NOP_OK) rc = CLB_NOP_ERR_CUDA;
+    cudaEventDestroy(ev);
+    return rc;
 }

@@ -43,6 +43,12 @@ class AdamSeg(ctypes.Structure):
                 ("rows", ctypes.c_int32), ("cols", ctypes.c_int32)]
 
 
+class NopLayer(ctypes.Structure):
+    """clb_nop_layer of include/clb_nop.h."""
+    _fields_ = [("w", _VP), ("wt", _VP), ("bias", _VP), ("cin", ctypes.c_int32), ("cout", ctypes.c_int32),
+                ("taps", ctypes.c_int32), ("relu", ctypes.c_int32)]
+
+
 def _lib():
     L = clb.load()
     if not getattr(L, "_nop_ready", False):
@@ -64,6 +70,15 @@ def _lib():
         L.clb_nop_check.argtypes = [_VP]
         L.clb_nop_wait_selftest.argtypes = [i64, _VP]
         L.clb_nop_add_mask.argtypes = [_VP, _VP, _VP, _VP, i64, _VP]
+        L.clb_nop_net_acts.argtypes = [ctypes.POINTER(NopLayer), i32, i32, i32, ctypes.POINTER(i64)]
+        L.clb_nop_net_acts.restype = i64
+        L.clb_nop_net_forward.argtypes = [ctypes.POINTER(NopLayer), _VP, i32, _VP, _VP, i32, i32, i32, _VP]
+        L.clb_nop_net_forward.restype = ctypes.c_int
+        L.clb_nop_net_scratch.argtypes = [ctypes.POINTER(NopLayer), i32, i32, i32]
+        L.clb_nop_net_scratch.restype = i64
+        pvp = ctypes.POINTER(_VP)
+        L.clb_nop_net_backward.argtypes = [ctypes.POINTER(NopLayer), pvp, pvp, pvp, _VP, _VP, i32, i32, i32, _VP, _VP]
+        L.clb_nop_net_backward.restype = ctypes.c_int
         L._nop_ready = True
     return L
 
@@ -240,7 +255,6 @@ class Net:
         layers.append(Conv(torch, r(c1), P(c1), cout, 1, False, rng, pad_out=False))
         net = cls(layers, torch)
         net.n_in = cin
-        net._zeros = {}
         net._flat_grads()
         return net
 
@@ -280,147 +294,60 @@ class Net:
             tot += one * (2 if i == 0 else 3)
         return tot
 
-    # ---- building blocks (all on the library's kernels)
-    def _conv(self, l, x, n, h, w, out_f32=False):
-        t = self.torch
-        y = t.empty((n, h, w, l.cout), dtype=t.float32 if out_f32 else t.bfloat16, device="cuda")
-        _ok(_lib().clb_nop_conv_fwd(_p(x), _p(l.wb), _p(l.wbt), _p(l.b), _p(y), int(out_f32), int(l.relu), n, h, w,
-                                    l.cin, l.cout, l.taps, None), "conv_fwd")
-        return y
+    # activations the forward pass keeps, in the library's order: name (a number:
+    # the output of that layer), the layer whose channel count it has (in: its
+    # input's), resolution divisor
+    ACTS = (("x", 0, True, 1), (1, 0, False, 1), (2, 1, False, 1), ("p1", 1, False, 2), (3, 2, False, 2), (4, 3, False, 2),
+            ("p2", 3, False, 4), (5, 4, False, 4), (6, 5, False, 4), ("p3", 5, False, 8), (7, 6, False, 8), (8, 7, False, 8),
+            ("c3", 8, True, 4), (9, 8, False, 4), (10, 9, False, 4), ("c2", 10, True, 2), (11, 10, False, 2),
+            (12, 11, False, 2), ("c1", 12, True, 1), (13, 12, False, 1), (14, 13, False, 1))
 
-    def _pool(self, x, n, h, w, c):
-        y = self.torch.empty((n, h // 2, w // 2, c), dtype=self.torch.bfloat16, device="cuda")
-        _ok(_lib().clb_nop_pool2(_p(x), _p(y), n, h, w, c, 0, None), "pool")
-        return y
+    def _table(self):
+        """The library's layer table, rebuilt when a layer's tensors have moved."""
+        key = [(_p(l.wb), _p(l.wbt), _p(l.b)) for l in self.layers]
+        if getattr(self, "_tab_key", None) != key:
+            self._tab = (NopLayer * len(self.layers))(*[NopLayer(*k, l.cin, l.cout, l.taps, int(l.relu))
+                                                        for k, l in zip(key, self.layers)])
+            self._tab_key = key
+        return self._tab
 
-    def _up(self, x, n, h, w, c):
-        y = self.torch.empty((n, 2 * h, 2 * w, c), dtype=self.torch.bfloat16, device="cuda")
-        _ok(_lib().clb_nop_up2(_p(x), _p(y), n, h, w, c, 0, None), "up")
-        return y
-
-    def _cat(self, a, b, npix, ca, cb):
-        y = self.torch.empty((npix, ca + cb), dtype=self.torch.bfloat16, device="cuda")
-        _ok(_lib().clb_nop_concat(_p(a), _p(b), _p(y), npix, ca, cb, 0, None), "concat")
-        return y
-
-    def _pad_input(self, x, n, h, w):
-        """(n, h, w, 8) -> (n, h, w, 32): the features and zero channels."""
-        t, npix = self.torch, n * h * w
-        pad = self.layers[0].cin - self.n_in
-        z = self._zeros.get(npix)
-        if z is None:
-            z = self._zeros[npix] = t.zeros((npix, pad), dtype=t.bfloat16, device="cuda")
-        y = t.empty((n, h, w, self.layers[0].cin), dtype=t.bfloat16, device="cuda")
-        _ok(_lib().clb_nop_concat(_p(x), _p(z), _p(y), npix, self.n_in, pad, 0, None), "pad")
-        return y
+    def _run(self, x, n, h, w):
+        """The forward pass by one library call: (output, buffer of all activations, their offsets)."""
+        t, lib, tab = self.torch, _lib(), self._table()
+        off = (ctypes.c_int64 * len(self.ACTS))()
+        size = lib.clb_nop_net_acts(tab, n, h, w, off)
+        if size <= 0:
+            raise RuntimeError(f"the network does not take {n} images of {h} x {w}")
+        buf = t.empty(size // 2, dtype=t.bfloat16, device="cuda")
+        out = t.empty((n, h, w, self.layers[-1].cout), dtype=t.float32, device="cuda")
+        _ok(lib.clb_nop_net_forward(tab, _p(x), self.n_in, _p(buf), _p(out), n, h, w, None), "net_forward")
+        return out, buf, off
 
     def forward(self, x, n, h, w):
         """x: (n, h, w, 8) BF16 device tensor -> (n, h, w, 4) FP32, plus the
         activations the backward pass needs (channels padded to multiples of 32)."""
-        L = self.layers
-        c1, c2, c3, c4 = L[0].cout, L[2].cout, L[4].cout, L[6].cout
-        x = self._pad_input(x, n, h, w)
-        A = {"x": x}
-        A[1] = self._conv(L[0], x, n, h, w)
-        A[2] = self._conv(L[1], A[1], n, h, w)
-        A["p1"] = self._pool(A[2], n, h, w, c1)
-        A[3] = self._conv(L[2], A["p1"], n, h // 2, w // 2)
-        A[4] = self._conv(L[3], A[3], n, h // 2, w // 2)
-        A["p2"] = self._pool(A[4], n, h // 2, w // 2, c2)
-        A[5] = self._conv(L[4], A["p2"], n, h // 4, w // 4)
-        A[6] = self._conv(L[5], A[5], n, h // 4, w // 4)
-        A["p3"] = self._pool(A[6], n, h // 4, w // 4, c3)
-        A[7] = self._conv(L[6], A["p3"], n, h // 8, w // 8)
-        A[8] = self._conv(L[7], A[7], n, h // 8, w // 8)
-        A["u3"] = self._up(A[8], n, h // 8, w // 8, c4)
-        A["c3"] = self._cat(A["u3"], A[6], n * (h // 4) * (w // 4), c4, c3)
-        A[9] = self._conv(L[8], A["c3"], n, h // 4, w // 4)
-        A[10] = self._conv(L[9], A[9], n, h // 4, w // 4)
-        A["u2"] = self._up(A[10], n, h // 4, w // 4, c3)
-        A["c2"] = self._cat(A["u2"], A[4], n * (h // 2) * (w // 2), c3, c2)
-        A[11] = self._conv(L[10], A["c2"], n, h // 2, w // 2)
-        A[12] = self._conv(L[11], A[11], n, h // 2, w // 2)
-        A["u1"] = self._up(A[12], n, h // 2, w // 2, c2)
-        A["c1"] = self._cat(A["u1"], A[2], n * h * w, c2, c1)
-        A[13] = self._conv(L[12], A["c1"], n, h, w)
-        A[14] = self._conv(L[13], A[13], n, h, w)
-        out = self._conv(L[14], A[14], n, h, w, out_f32=True)
+        out, buf, off = self._run(x, n, h, w)
+        A = {}
+        for (name, l, is_in, d), o in zip(self.ACTS, off):
+            c = self.layers[l].cin if is_in else self.layers[l].cout
+            shape = (n, h // d, w // d, c)
+            A[name] = buf[o // 2:o // 2 + math.prod(shape)].view(shape)
         return out, A
 
     # ---- backward
-    def _grads(self, l, x, dy, n, h, w, mask, want_dx=True):
-        """Accumulate l's weight and bias gradients; return dx (BF16) masked
-        by `mask` > 0 (the ReLU of the layer that produced x) if given.  The
-        weight gradient, which nothing before the optimiser step needs, runs
-        on a side stream, overlapping the input-gradient chain of the
-        default stream."""
-        lib, t = _lib(), self.torch
-        ev = t.cuda.Event()
-        ev.record(t.cuda.default_stream())
-        self._ws.wait_event(ev)
-        _ok(lib.clb_nop_conv_wgrad_bias(_p(x), _p(dy), _p(l.gw), _p(l.gb), n, h, w, l.cin, l.cout, l.taps, 0,
-                                        _VP(self._ws.cuda_stream)), "wgrad")
-        x.record_stream(self._ws)
-        dy.record_stream(self._ws)
-        if not want_dx:
-            return None
-        dx = t.empty((n, h, w, l.cin), dtype=t.bfloat16, device="cuda")
-        _ok(lib.clb_nop_conv_dgrad(_p(dy), _p(l.wb), _p(mask), _p(dx), n, h, w, l.cin, l.cout, l.taps, None),
-            "dgrad")
-        return dx
-
-    def _split(self, y, npix, ca, cb):
-        t = self.torch
-        a = t.empty((npix, ca), dtype=t.bfloat16, device="cuda")
-        b = t.empty((npix, cb), dtype=t.bfloat16, device="cuda")
-        _ok(_lib().clb_nop_concat(_p(a), _p(b), _p(y), npix, ca, cb, 1, None), "split")
-        return a, b
-
-    def _add_mask(self, d1, d2, a):
-        out = self.torch.empty_like(d1)
-        _ok(_lib().clb_nop_add_mask(_p(d1), _p(d2), _p(a), _p(out), d1.numel(), None), "add_mask")
-        return out
-
     def backward(self, dout, A, n, h, w):
-        L, t, lib = self.layers, self.torch, _lib()
-        c1, c2, c3, c4 = L[0].cout, L[2].cout, L[4].cout, L[6].cout
+        """Accumulates every layer's weight and bias gradient (cleared first)
+        from the gradient of the output and the activations of forward()."""
+        t, lib, tab = self.torch, _lib(), self._table()
         if getattr(self, "_ws", None) is None:
-            self._ws = t.cuda.Stream()
+            self._ws = t.cuda.Stream()      # the weight gradients run beside the input-gradient chain
         _ok(lib.clb_nop_zero(_p(self.grads), self.grads.numel() * 4, None), "zero")
-        h2, w2, h4, w4, h8, w8 = h // 2, w // 2, h // 4, w // 4, h // 8, w // 8
-        d = self._grads(L[14], A[14], dout, n, h, w, A[14])
-        d = self._grads(L[13], A[13], d, n, h, w, A[13])
-        dc1 = self._grads(L[12], A["c1"], d, n, h, w, None)
-        du1, d2_skip = self._split(dc1, n * h * w, c2, c1)
-        d12 = t.empty((n, h2, w2, c2), dtype=t.bfloat16, device="cuda")
-        _ok(lib.clb_nop_up2(_p(du1), _p(d12), n, h2, w2, c2, 1, None), "up_bwd")
-        d = self._grads(L[11], A[11], self._add_mask(d12, None, A[12]), n, h2, w2, A[11])
-        dc2 = self._grads(L[10], A["c2"], d, n, h2, w2, None)
-        du2, d4_skip = self._split(dc2, n * h2 * w2, c3, c2)
-        d10 = t.empty((n, h4, w4, c3), dtype=t.bfloat16, device="cuda")
-        _ok(lib.clb_nop_up2(_p(du2), _p(d10), n, h4, w4, c3, 1, None), "up_bwd")
-        d = self._grads(L[9], A[9], self._add_mask(d10, None, A[10]), n, h4, w4, A[9])
-        dc3 = self._grads(L[8], A["c3"], d, n, h4, w4, None)
-        du3, d6_skip = self._split(dc3, n * h4 * w4, c4, c3)
-        d8 = t.empty((n, h8, w8, c4), dtype=t.bfloat16, device="cuda")
-        _ok(lib.clb_nop_up2(_p(du3), _p(d8), n, h8, w8, c4, 1, None), "up_bwd")
-        d = self._grads(L[7], A[7], self._add_mask(d8, None, A[8]), n, h8, w8, A[7])
-        dp3 = self._grads(L[6], A["p3"], d, n, h8, w8, None)
-        d6 = t.empty((n, h4, w4, c3), dtype=t.bfloat16, device="cuda")
-        _ok(lib.clb_nop_pool2(_p(dp3), _p(d6), n, h4, w4, c3, 1, None), "pool_bwd")
-        d = self._grads(L[5], A[5], self._add_mask(d6, d6_skip, A[6]), n, h4, w4, A[5])
-        dp2 = self._grads(L[4], A["p2"], d, n, h4, w4, None)
-        d4 = t.empty((n, h2, w2, c2), dtype=t.bfloat16, device="cuda")
-        _ok(lib.clb_nop_pool2(_p(dp2), _p(d4), n, h2, w2, c2, 1, None), "pool_bwd")
-        d = self._grads(L[3], A[3], self._add_mask(d4, d4_skip, A[4]), n, h2, w2, A[3])
-        dp1 = self._grads(L[2], A["p1"], d, n, h2, w2, None)
-        d2 = t.empty((n, h, w, c1), dtype=t.bfloat16, device="cuda")
-        _ok(lib.clb_nop_pool2(_p(dp1), _p(d2), n, h, w, c1, 1, None), "pool_bwd")
-        d = self._grads(L[1], A[1], self._add_mask(d2, d2_skip, A[2]), n, h, w, A[1])
-        self._grads(L[0], A["x"], d, n, h, w, None, want_dx=False)
-        done = t.cuda.Event()                 # the optimiser step waits for every weight gradient
-        done.record(self._ws)
-        t.cuda.default_stream().wait_event(done)
+        nl = len(self.layers)
+        gw, gb = (_VP * nl)(*[_p(l.gw) for l in self.layers]), (_VP * nl)(*[_p(l.gb) for l in self.layers])
+        acts = (_VP * len(self.ACTS))(*[_p(A[name]) for name, *_ in self.ACTS])
+        scratch = t.empty(lib.clb_nop_net_scratch(tab, n, h, w) // 2, dtype=t.bfloat16, device="cuda")
+        _ok(lib.clb_nop_net_backward(tab, gw, gb, acts, _p(dout), _p(scratch), n, h, w, None,
+                                     _VP(self._ws.cuda_stream)), "net_backward")
 
     def adam(self, step, lr, b1=0.9, b2=0.999, eps=1e-8):
         # one launch: every layer's weights (BF16 copy and its transpose refreshed) and biases
@@ -514,9 +441,8 @@ def predict(net: Net, X: np.ndarray, batch: int = 16) -> np.ndarray:
     outs = []
     for b in range(0, n, batch):
         xb = to_bf16(torch, X[b:b + batch])
-        out, _ = net.forward(xb, xb.shape[0], h, w)
-        outs.append(out.cpu().numpy())
-    return np.concatenate(outs, axis=0)
+        outs.append(net._run(xb, xb.shape[0], h, w)[0].cpu().numpy())
+    return np.concatenate(outs, axis=0) if len(outs) != 1 else outs[0]
 
 
 def warm_fields(net: Net, phi: np.ndarray, Ra: float, Da: float, Pr: float, sigma: float):
