@@ -1434,7 +1434,8 @@ __device__ __forceinline__ bool split_step_wall(const BufT<double>& in, const Bu
 #pragma unroll
         for (int i = 0; i < 5; ++i) n0ss += fix_g(L::ld(in.g + i * G.plane + o[i]), P.gexp, big);
     }
-    const bool ok = split_wall<SHIFT, FORCH>(f, g, n0ss, cs, cb, w.su, w.st, P);
+    const bool ok = P.rest[w.su] ? split_wall<SHIFT, FORCH, true>(f, g, n0ss, cs, cb, w.su, w.st, P)
+                                 : split_wall<SHIFT, FORCH, false>(f, g, n0ss, cs, cb, w.su, w.st, P);
     if (!(ok && fix_ok(range) && big < P.gmax)) return false;
     split_store(out, G, P, x, y, f, g);
     return true;

@@ -286,6 +286,7 @@ struct SplitPhys {
     uint32_t gmax;                   // high word of 2^gexp: |g| stays below it
     sf uw[4], vw[4], Tw[4];          // walls: velocity, temperature (units of 2^gexp)
     long long n0w[4], cw[4];         // and sigma T_w, c_sT^2 T_w in fixed point
+    int rest[4];                     // the wall does not move
 };
 
 // The constants of a run.  top: the largest temperature the run starts with
@@ -335,6 +336,7 @@ inline SplitPhys split_phys(double sp, double sm, double sv, double s3, double s
         const double T = fits && iso[s] ? ldexp(Tw[s], -e) : 0.0;
         P.uw[s] = sf_make(uw[s]);
         P.vw[s] = sf_make(vw[s]);
+        P.rest[s] = uw[s] == 0.0 && vw[s] == 0.0;
         P.Tw[s] = sf_make(T);
         P.n0w[s] = llrint(ldexp(sigma * T, 60));
         P.cw[s] = llrint(ldexp(cT2 * T, 60));
@@ -548,7 +550,9 @@ CLB_SP bool split_node(long long (&f)[9], long long (&g)[5], const SplitCoef& c,
 // node's post-collision values out.  side_u: the wall that sets the velocity;
 // side_t: the isothermal wall that sets the temperature, or -1 (adiabatic:
 // n0ss = sum g of the next node inward).
-template <bool SHIFT, bool FORCH>
+// REST: the wall does not move (both velocities 0), the usual case; what
+// vanishes then is left out (the wall nodes are a small grid's longest chain).
+template <bool SHIFT, bool FORCH, bool REST>
 CLB_SP bool split_wall(long long (&f)[9], long long (&g)[5], long long n0ss, const SplitCoef& cs, const SplitCoef& cb,
                        int side_u, int side_t, const SplitPhys& P) {
     const FixMom k = fix_moments(f);
@@ -572,10 +576,16 @@ CLB_SP bool split_wall(long long (&f)[9], long long (&g)[5], long long n0ss, con
     }
     float worst = 0.0f;
     // temperature: d = g+ - g- at b is its value at s plus T_b u_w - T_s u_s
-    const sf2 TU = mul(both(Tn), uw), t = fnma(both(Tsn), U, TU);
     const long long D1 = g[1] - g[3], D2 = g[2] - g[4];
-    long long qs[2], qv[2];
-    const sf2 v = dbl(add(split_axes<SHIFT>(TU, add(to_sf2(D1, D2), t), uw, P, qs, worst), t));
+    long long qs[2] = {0, 0}, qv[2];
+    sf2 v;
+    if constexpr (REST) {   // T_b u_w = 0: s = 0, 2 b = -zeta_a d
+        const sf2 t = neg(mul(both(Tsn), U));
+        v = dbl(fnma(both(dbl(P.hza)), add(to_sf2(D1, D2), t), t));
+    } else {
+        const sf2 TU = mul(both(Tn), uw), t = fnma(both(Tsn), U, TU);
+        v = dbl(add(split_axes<SHIFT>(TU, add(to_sf2(D1, D2), t), uw, P, qs, worst), t));
+    }
     worst = fabs_max(worst, v.h.x, v.h.y);
     to_fix4(v, qv[0], qv[1]);
     const long long e1 = C + (qs[0] << 2), e2 = C + (qs[1] << 2);
@@ -584,23 +594,46 @@ CLB_SP bool split_wall(long long (&f)[9], long long (&g)[5], long long n0ss, con
     g[3] = e1 - g[1];
     g[2] = (e2 + D2 + (qv[1] << 1)) >> 1;
     g[4] = e2 - g[2];
-    // flow: moments of b minus those of s
-    const sf2 RU = mul(both(rho), U), IU = mul(both(cs.ip), U), ru = mul(both(rho), uw), iu = mul(both(cb.ip), uw);
-    const sf sXY = mul(first(IU), second(RU)), wXY = mul(first(iu), second(ru));
-    const sf2 m34 = sub(mul(iu, ru), mul(IU, RU));
-    const sf m5 = sub(wXY, sXY);
-    const sf2 m67 = sub(mul(both(wXY), uw), mul(both(sXY), U));
-    const sf m8 = fma(P.third, sum(m34), sub(mul(wXY, mul(first(iu), second(uw))), mul(sXY, mul(first(IU), second(U)))));
+    // flow: moments of b minus those of s, and the collision's increments at b
     SplitMom m = split_moments(k, P);
-    m.a34 = add(m.a34, m34);
-    m.a67 = add(m.a67, m67);
-    m.a5 = add(m.a5, m5);
-    m.a8 = add(m.a8, m8);
-    const sf2 Fb = mul(both(rho), split_force<FORCH>(uw, scale(Tn, P.tunit), cb));
-    Incr8 r = split_collide<SHIFT, false>(m, rho, uw, p, Fb, cb.ip, P);
+    sf2 m34, ru;
+    sf m5, m8;
+    Incr8 r;
+    const sf2 RU = mul(both(rho), U), IU = mul(both(cs.ip), U);
+    const sf sXY = mul(first(IU), second(RU)), sq = mul(sXY, mul(first(IU), second(U)));
+    if constexpr (REST) {
+        m34 = neg(mul(IU, RU));
+        m5 = neg(sXY);
+        m8 = sub(mul(P.third, sum(m34)), sq);
+        m.a34 = add(m.a34, m34);
+        m.a67 = fnma(both(sXY), U, m.a67);
+        m.a5 = add(m.a5, m5);
+        m.a8 = add(m.a8, m8);
+        const sf2 F = mul(both(rho), pair(cb.hgx, fma(cb.hgb, scale(Tn, P.tunit), cb.hgy)));
+        r.r12 = add(p, F);
+        r.r34 = neg(fma(both(P.sp), m.a34, mul(both(P.sm), swp(m.a34))));
+        r.r5 = neg(mul(P.sv, m.a5));
+        // shift and unit shift agree at u = 0: -s3 (k21 - rho u_y / 3) + (1 - s3 / 2) rho F_y / 3
+        r.r67 = fms(both(P.c62), swp(F), mul(both(P.s3), fnma(both(P.third), swp(p), m.a67)));
+        r.r8 = neg(mul(P.s4, m.a8));
+    } else {
+        ru = mul(both(rho), uw);
+        const sf2 iu = mul(both(cb.ip), uw);
+        const sf wXY = mul(first(iu), second(ru));
+        m34 = sub(mul(iu, ru), mul(IU, RU));
+        m5 = sub(wXY, sXY);
+        m8 = fma(P.third, sum(m34), sub(mul(wXY, mul(first(iu), second(uw))), sq));
+        m.a34 = add(m.a34, m34);
+        m.a67 = add(m.a67, sub(mul(both(wXY), uw), mul(both(sXY), U)));
+        m.a5 = add(m.a5, m5);
+        m.a8 = add(m.a8, m8);
+        const sf2 Fb = mul(both(rho), split_force<FORCH>(uw, scale(Tn, P.tunit), cb));
+        r = split_collide<SHIFT, false>(m, rho, uw, p, Fb, cb.ip, P);
+    }
     // increments against s: the first-order rows and j / 3 of rows 6, 7 are
     // replaced outright (their values at s go out in fixed point)
-    const sf2 j = sub(ru, p);
+    sf2 j = neg(p);
+    if constexpr (!REST) j = sub(ru, p);
     r.r12 = add(r.r12, j);
     r.r34 = add(r.r34, m34);
     r.r5 = add(r.r5, m5);

@@ -1512,6 +1512,8 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    pdl_start();   // every CTA holds its TMEM (see k_conv_tma)
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
 
     // Both issuers walk the same items: for every run of rows [ya, yb) within
@@ -1963,8 +1965,8 @@ bool launch_wgrad_row(const void* x, const void* dy, float* dw, float* db, ConvS
         *rc = CLB_NOP_ERR_CUDA;
         return true;
     }
-    k_wgrad_row<<<dim3((unsigned)groups, (unsigned)ntn, (unsigned)gz), TC_THREADS, smem, st>>>(
-        mx, my, dw, db, s, atoms, na, bw, tile_n, cols, stages, x_bytes, y_bytes);
+    launch_pdl(k_wgrad_row, dim3((unsigned)groups, (unsigned)ntn, (unsigned)gz), TC_THREADS, smem, st, mx, my, dw, db, s, atoms,
+               na, bw, tile_n, cols, stages, x_bytes, y_bytes);
     *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     return true;
 }
@@ -2973,19 +2975,32 @@ extern "C" int clb_nop_net_backward(const clb_nop_layer* L, float* const* gw, fl
     auto G = [&](int i) -> void* { return (char*)scratch + off[i]; };
     const int res[kNetLayers] = {1, 1, 2, 2, 4, 4, 8, 8, 4, 4, 2, 2, 1, 1, 1};
     int rc = CLB_NOP_OK;
-    // Layer l: weight and bias gradient on the side stream (nothing before the
-    // optimiser needs them), then the input gradient on the main one.
+    // Layer l: the input gradient on the main stream; its weight and bias
+    // gradients, which nothing before the optimiser needs, on the side stream.
+    // Those go there a few layers at a time: an event between two of them would
+    // keep the second's launch from overlapping the first (about 8 us each).
+    struct {
+        int l, in;
+        const void* dy;
+    } pend[kNetLayers];
+    int np = 0;
+    auto flush = [&]() {
+        if (rc == CLB_NOP_OK && np && (cudaEventRecord(ev, st) != cudaSuccess || cudaStreamWaitEvent(side, ev, 0) != cudaSuccess))
+            rc = CLB_NOP_ERR_CUDA;
+        for (int k = 0; k < np && rc == CLB_NOP_OK; ++k) {
+            const int l = pend[k].l;
+            rc = clb_nop_conv_wgrad_bias(acts[pend[k].in], pend[k].dy, gw[l], gb[l], n, h / res[l], w / res[l], L[l].cin, L[l].cout,
+                                         L[l].taps, 0, side_stream);
+        }
+        np = 0;
+    };
     auto layer = [&](int l, int in, const void* dy, bool masked) {
         if (rc != CLB_NOP_OK) return;
-        const int hh = h / res[l], ww = w / res[l];
-        if (cudaEventRecord(ev, st) != cudaSuccess || cudaStreamWaitEvent(side, ev, 0) != cudaSuccess) {
-            rc = CLB_NOP_ERR_CUDA;
-            return;
-        }
-        rc = clb_nop_conv_wgrad_bias(acts[in], dy, gw[l], gb[l], n, hh, ww, L[l].cin, L[l].cout, L[l].taps, 0, side_stream);
+        pend[np++] = {l, in, dy};
+        if (l == 13 || l == 11 || l == 9 || l == 6 || l == 3 || l == 1 || l == 0) flush();
         if (rc == CLB_NOP_OK && l > 0)
-            rc = clb_nop_conv_dgrad(dy, L[l].w, masked ? acts[in] : nullptr, G(l - 1), n, hh, ww, L[l].cin, L[l].cout, L[l].taps,
-                                    stream);
+            rc = clb_nop_conv_dgrad(dy, L[l].w, masked ? acts[in] : nullptr, G(l - 1), n, h / res[l], w / res[l], L[l].cin, L[l].cout,
+                                    L[l].taps, stream);
     };
     // d a (at 1/d of the resolution) from the gradient of [up(a) | skip] at 2/d
     auto up = [&](const void* dc, int act, int slot, int d, int ca, int cb) {
