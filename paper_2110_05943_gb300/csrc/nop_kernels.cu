@@ -523,10 +523,7 @@ constexpr int TM_THREADS = 320;
 #define CLB_ROW_MAX_STAGES 6
 #endif
 #ifndef CLB_WR_MAX_STAGES
-#define CLB_WR_MAX_STAGES 5
-#endif
-#ifndef CLB_WR_CTAS
-#define CLB_WR_CTAS 1
+#define CLB_WR_MAX_STAGES 10
 #endif
 constexpr int TM_BIAS_MAX = 1024;                // outputs whose bias is staged in shared memory
 
@@ -1444,17 +1441,25 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tma(const __grid_constant_
 // row at a time: D[(tap, c)][n] = sum over pixels p of X[p + d(tap)][c] dY[p][n].
 // k_wgrad_tma fetches the activations once per tap (nine boxes per 64 pixels,
 // and each of its M tiles fetches dY again); its copies' request rate set the
-// pace.  Here a row of X, with one pixel of halo on either side, and the row of
-// dY below it are fetched once, into one stage of a ring; the three newest X
-// rows serve the taps dy = -1, 0, 1, and the taps dx = -1, 0, 1 are the same
-// bytes one pixel further on: both operands are MN-major (pixels along K), so
-// the M = 128 rows of an MMA are four 32-channel atoms whose leading byte
-// offset is one pixel (64 bytes; the swizzle follows the address).  The
-// fourth (dx = 2) is not stored.  Accumulators: a tile of tile_n columns per
-// (atom, dy), and with db one more whose A operand is a column of ones (its row
-// 0 is the bias gradient).  Rows are split over gridDim.z; gridDim.x takes
-// groups of `na` atoms, gridDim.y the output tiles.  16 x 128^2, 32 -> 32: 58.5
-// us before; see the launcher for the shapes.
+// pace.  Here every row is fetched once, into a ring: dY row y + 1 and, with a
+// pixel of halo on either side, X row y.  The taps are views of the same bytes:
+//   dx  the operands are MN-major (pixels along K), so the M = 128 rows of an
+//       MMA are four 32-channel atoms of X whose leading byte offset is one
+//       pixel (64 bytes; the swizzle follows the address).  The fourth (dx = 2)
+//       is not stored.
+//   dy  the N columns are those of up to three dY rows, neighbours in the ring
+//       (dY rows y - 1, y, y + 1 meet X row y at the taps dy = 1, 0, -1); two
+//       MMAs where the ring wraps between them or three rows exceed N = 256.
+// The thread that issues the MMAs bounds this kernel (it took the same time
+// without its copies, and half without its MMAs), hence few wide MMAs and a loop
+// over constant offsets (wr_row).  A first form kept three X rows and took an MMA
+// per (atom, dy), N = tile_n: 16 x 128^2, 32 -> 32: 31.8 us, 96 -> 32: 56.3; with
+// one MMA per atom 23.9 and 43.8; with the loop unrolled 17.3 and 32.6; with a
+// ring of up to ten stages, so that fewer rows wrap, 16.5 and 32.5.
+// The bias gradient: a column of ones as A; the N columns are those of `bm`
+// successive 16-pixel steps of dY row y (128 columns in all), added up at the end.
+// Rows are split over gridDim.z; gridDim.x takes groups of `na` atoms, gridDim.y
+// the output tiles.
 //   thread 0: copies, ring of `stages`; thread 32: MMAs; then warp j < 3 adds
 //   its rows (tap dx = j - 1) to dw with 16-byte reductions.
 // Every wait is bounded, as in k_conv_tma.
@@ -1462,6 +1467,24 @@ constexpr int WR_ONES = 16 * 64;   // bytes of the ones operand: 16 K rows of 64
 
 __device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+// The MMAs of one X row: `ksteps` steps of 16 pixels, NC atoms, in one or two
+// column groups (the second starts at column d2).
+template <int NC, bool TWO>
+__device__ __forceinline__ void wr_row(uint32_t tmem, uint32_t al, uint32_t b1, uint32_t b2, uint32_t bhi, uint32_t id1,
+                                       uint32_t id2, int tile_n, uint32_t d2, uint32_t xj, int bstep, int ksteps,
+                                       uint32_t acc) {
+#pragma unroll 2
+    for (int ks = 0; ks < ksteps; ++ks) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            const uint32_t d = tmem + (uint32_t)(3 * tile_n * j), a = al + (uint32_t)(64 * ks) + xj * j;
+            tc_mma_lo(d, a, desc_hi(64), b1 + (uint32_t)(bstep * ks), bhi, id1, acc);
+            if (TWO) tc_mma_lo(d + d2, a, desc_hi(64), b2 + (uint32_t)(bstep * ks), bhi, id2, acc);
+        }
+        acc = 1;
+    }
 }
 
 __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant__ CUtensorMap mapX,
@@ -1473,8 +1496,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
     unsigned char* const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const int atom0 = blockIdx.x * na, nc = min(na, atoms - atom0), n0 = blockIdx.y * tile_n;
     const int nby = tile_n / bw;
-    const int stage_bytes = na * x_bytes + nby * y_bytes;          // both multiples of 1024
-    unsigned char* const ones = smem + stages * stage_bytes;       // 1024 bytes
+    const int xs = na * x_bytes, ys = nby * y_bytes;               // of one stage; multiples of 1024
+    unsigned char* const ysm = smem + stages * xs;                 // the dY rows, one after the other
+    unsigned char* const ones = ysm + stages * ys;                 // 1024 bytes
     uint64_t* full = reinterpret_cast<uint64_t*>(ones + WR_ONES);
     uint64_t* empty = full + stages;
     uint64_t* done = empty + stages;
@@ -1485,6 +1509,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
     const int rows = s.n * s.h;
     const int r0 = (int)((long long)rows * blockIdx.z / gridDim.z), r1 = (int)((long long)rows * (blockIdx.z + 1) / gridDim.z);
     const bool bias = db && atom0 == 0;
+    const int ksteps = s.w / 16, bm = max(1, 128 / tile_n);
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -1517,7 +1542,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
     const uint32_t tmem = *tmem_slot;
 
     // Both issuers walk the same items: for every run of rows [ya, yb) within
-    // an image, X rows ya - 1 .. yb, and with X row y + 1 the dY row y.
+    // an image, dY rows ya - 1 .. yb, and with dY row y + 1 the X row y.
     bool ok = true;
     if (tid == 0) {   // copies
         int it = 0, st = 0, ph = 0;
@@ -1529,12 +1554,11 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
                     break;
                 }
                 const int y = x - 1;
-                const uint32_t fb = smem_u32(&full[st]), base = smem_u32(smem + st * stage_bytes);
-                mbar_expect_tx(fb, (uint32_t)(nc * (s.w + 2) * 64 + (y >= ya ? nby * s.w * bw * 2 : 0)));
-                for (int j = 0; j < nc; ++j) tma_load_4d(base + j * x_bytes, &mapX, fb, (atom0 + j) * 32, -1, x, img);
+                const uint32_t fb = smem_u32(&full[st]), xb = smem_u32(smem + st * xs), yr = smem_u32(ysm + st * ys);
+                mbar_expect_tx(fb, (uint32_t)(nby * s.w * bw * 2 + (y >= ya ? nc * (s.w + 2) * 64 : 0)));
+                for (int j = 0; j < nby; ++j) tma_load_4d(yr + j * y_bytes, &mapY, fb, n0 + j * bw, 0, x, img);
                 if (y >= ya)
-                    for (int j = 0; j < nby; ++j)
-                        tma_load_4d(base + na * x_bytes + j * y_bytes, &mapY, fb, n0 + j * bw, 0, y, img);
+                    for (int j = 0; j < nc; ++j) tma_load_4d(xb + j * x_bytes, &mapX, fb, (atom0 + j) * 32, -1, y, img);
                 ++it;
                 if (++st == stages) {
                     st = 0;
@@ -1545,10 +1569,13 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
         }
         s_issued = it;
     } else if (tid == 32) {   // MMAs
-        const uint32_t idesc = tc_idesc(tile_n) | (1u << 15) | (1u << 16);   // A and B MN-major
-        const uint32_t ring_lo = desc_lo(smem_u32(smem), 64), ones_lo = desc_lo(smem_u32(ones), 0);
-        const uint32_t by_lo = desc_lo(smem_u32(smem) + na * x_bytes, (uint32_t)y_bytes), bhi = desc_hi(2 * bw);
-        const int stage_lo = stage_bytes >> 4;
+        const uint32_t mn = (1u << 15) | (1u << 16);   // A and B MN-major
+        const uint32_t x_lo = desc_lo(smem_u32(smem), 64), ones_lo = desc_lo(smem_u32(ones), 0);
+        const uint32_t y_lo = desc_lo(smem_u32(ysm), (uint32_t)y_bytes), bhi = desc_hi(2 * bw);
+        // the next 16 pixels as the next columns (one step at a time where a row is several atoms wide)
+        const uint32_t bias_lo = nby > 1 ? y_lo : desc_lo(smem_u32(ysm), (uint32_t)(32 * bw));
+        const uint32_t d_bias = tmem + (uint32_t)(3 * na * tile_n);
+        const int maxr = min(3, 256 / tile_n);
         int it = 0, st = 0, ph = 0;
         uint32_t acc = 0;
         for (int r = r0; r < r1 && ok;) {
@@ -1561,23 +1588,30 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
                 }
                 if (x > ya) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t lo[3] = {ring_lo + (uint32_t)(p2 * stage_lo), ring_lo + (uint32_t)(p1 * stage_lo),
-                                            ring_lo + (uint32_t)(st * stage_lo)};
-                    uint32_t bl = by_lo + (uint32_t)(st * stage_lo);
-                    for (int ks = 0; ks < s.w / 16; ++ks) {
-                        uint32_t d = tmem;
-                        for (int j = 0; j < nc; ++j) {
-                            const uint32_t off = (uint32_t)(j * (x_bytes >> 4) + ks * 64);
-#pragma unroll
-                            for (int dy = 0; dy < 3; ++dy) {
-                                tc_mma_lo(d, lo[dy] + off, desc_hi(64), bl, bhi, idesc, acc);
-                                d += (uint32_t)tile_n;
-                            }
-                        }
-                        if (bias) tc_mma_lo(tmem + (uint32_t)(3 * na * tile_n), ones_lo, desc_hi(64), bl, bhi, idesc, acc);
-                        bl += (uint32_t)(2 * bw);
-                        acc = 1;
+                    // the first k1 of the three dY rows lie one after the other from p2 on
+                    const int k1 = min(maxr, st >= 2 ? 3 : 2 - st), q = p2 + k1 >= stages ? p2 + k1 - stages : p2 + k1;
+                    const uint32_t id1 = tc_idesc(k1 * tile_n) | mn, id2 = tc_idesc((3 - k1) * tile_n) | mn;
+                    const uint32_t al = x_lo + (uint32_t)(st * (xs >> 4));
+                    const uint32_t b1 = y_lo + (uint32_t)(p2 * (ys >> 4)), b2 = y_lo + (uint32_t)(q * (ys >> 4));
+                    const uint32_t d2 = (uint32_t)(k1 * tile_n), xj = (uint32_t)(x_bytes >> 4);
+                    if (k1 == 3) {
+                        if (nc == 1) wr_row<1, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                        else if (nc == 2) wr_row<2, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                        else if (nc == 3) wr_row<3, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                        else wr_row<4, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                    } else {
+                        if (nc == 1) wr_row<1, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                        else if (nc == 2) wr_row<2, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                        else if (nc == 3) wr_row<3, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                        else wr_row<4, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
                     }
+                    if (bias)
+                        for (int ks = 0; ks < ksteps; ks += bm) {
+                            tc_mma_lo(d_bias, ones_lo, desc_hi(64), bias_lo + (uint32_t)(p1 * (ys >> 4) + ks * 2 * bw), bhi,
+                                      tc_idesc(min(bm, ksteps - ks) * tile_n) | mn, acc);
+                            acc = 1;
+                        }
+                    acc = 1;
                     tc_commit(smem_u32(&empty[p2]));
                     if (x == yb) {   // the run's last rows are free too
                         tc_commit(smem_u32(&empty[p1]));
@@ -1609,13 +1643,21 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
         for (int q = 0; q < 3 * nc + (bias ? 1 : 0); ++q) {
             const bool is_bias = q == 3 * nc;
             const int col = (is_bias ? 3 * na : q) * tile_n;
-            const int tap = (q % 3) * 3 + warp, c = (atom0 + q / 3) * 32 + lane;
+            const int tap = (2 - q % 3) * 3 + warp, c = (atom0 + q / 3) * 32 + lane;
             float* dst = is_bias ? db + n0 : dw + (size_t)(tap * s.cin + c) * s.cout + n0;
             const bool live = is_bias ? tid == 0 : warp < 3;
             for (int c0 = 0; c0 < tile_n; c0 += 32) {
                 uint32_t v[32];
                 tc_ld32_nowait(lanes + (uint32_t)(col + c0), v);
                 tc_wait_ld();
+                if (is_bias)
+                    for (int m = 1; m < min(bm, ksteps); ++m) {
+                        uint32_t u[32];
+                        tc_ld32_nowait(lanes + (uint32_t)(col + m * tile_n + c0), u);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(u[j]));
+                    }
                 if (live)
 #pragma unroll
                     for (int j = 0; j < 32; j += 4)
@@ -1931,20 +1973,26 @@ bool launch_wgrad_row(const void* x, const void* dy, float* dw, float* db, ConvS
     const long long npix = (long long)s.n * s.h * s.w;
     if (npix * (s.cin > s.cout ? s.cin : s.cout) * s.taps >= 2147483647LL) return false;
     // output tile: the whole of narrow layers, else 64 or 32 columns; then as
-    // many atoms as their three accumulators and the bias's fit in TMEM
+    // many atoms as their three accumulators and the bias's columns fit in TMEM
     const int tile_n = s.cout <= 96 ? s.cout : s.cout % 64 == 0 ? 64 : 32;
     const int bw = tile_n % 64 == 0 ? 64 : 32;
-    const int atoms = s.cin / 32, na = std::min(atoms, (512 / tile_n - 1) / 3);
+    const int atoms = s.cin / 32, bcols = std::max(tile_n, 128);
+    const int na = std::min(atoms, (512 - bcols) / (3 * tile_n));
     const int groups = (atoms + na - 1) / na, ntn = s.cout / tile_n;
     int cols = 32;
-    while (cols < (3 * na + 1) * tile_n) cols <<= 1;
+    while (cols < 3 * na * tile_n + bcols) cols <<= 1;
     const int x_bytes = ((s.w + 3) * 64 + 1023) / 1024 * 1024, y_bytes = (s.w * bw * 2 + 1023) / 1024 * 1024;
     const size_t stage_bytes = (size_t)na * x_bytes + (size_t)(tile_n / bw) * y_bytes;
     const int stages = (int)std::min<size_t>(CLB_WR_MAX_STAGES, (200 * 1024) / stage_bytes);
     if (stages < 4) return false;
     const int rows = s.n * s.h;
-    long long gz = splitk >= 1 ? splitk : std::max(1, CLB_WR_CTAS * sm_count() / (groups * ntn));
-    gz = std::max(1LL, std::min(gz, splitk >= 1 ? (long long)rows : (long long)(rows + 3) / 4));
+    // one CTA per SM (two measured slower: 471 us against 407 over the network's
+    // layers), but enough rows in each to pay for adding its 9 x 32 na x tile_n
+    // sums to dw: 16 x 64^2, 64 -> 64: 24.0 us with 152 CTAs, 21.2 with 102
+    // (10 rows each), 22.2 with 50; 16 x 32^2, 64 -> 96: 15.5 with 152, 13.9 with 128
+    const int least = std::max(4, na * tile_n / 12);
+    long long gz = splitk >= 1 ? splitk : std::max(1, sm_count() / (groups * ntn));
+    gz = std::max(1LL, std::min(gz, splitk >= 1 ? (long long)rows : (long long)(rows + least - 1) / least));
     if (gz > 65535) return false;
     CUtensorMap mx, my;
     {
