@@ -61,18 +61,11 @@ WORKLOAD = ("{n}x{n} porous cavity, seeded GRF porosity 0.3+0.6*Phi(g) (l=32, se
 # Algorithmic bytes per coupled cell update of the FP64 form: 14 distribution
 # values read and 14 written (8 B each) plus the porosity (8 B).
 BYTES_PER_CCU_F64 = 28 * 8 + 8
-# FP64 floating-point operations per coupled cell update executed by the FP64
-# step kernel (dadd + dmul + 2 dfma per launch / nodes, ncu instruction
-# counters of the current kernel), and its FP64 pipe instructions (dadd +
-# dmul + dfma) per node.
-FP64_FLOP_PER_CCU = 257.5
-FP64_INST_PER_CCU = 175.4
 # DRAM bytes (read + write) per node of one launch of the current FP64 step
 # kernel, ncu on the 2048^2 case of the same workload, scaled by the node
 # count (traffic grows with the nodes): 14 + 14 values and the 64-byte
 # per-node constant table.
-DRAM_BYTES_PER_CCU_MEASURED = 282.7
-SMS, DFMA_PER_CLK_PER_SM = 152, 2   # GB300 FP64 pipe: 2 DFMA/clk/SM (1.25 TFLOP/s at 2.07 GHz)
+DRAM_BYTES_PER_CCU_MEASURED = 283.5
 
 
 def _peaks():
@@ -665,7 +658,6 @@ def _summary(line):
     r3 = lambda v: None if v is None else float(f"{v:.4g}")
     s = {f"f64_{line['config']['nx']}": {"mlups": r3(line["value"]), "frac": r3(line["roofline"]["frac"]),
                       "bound": line["roofline"]["bound"],
-                      "fp64_pipe_frac": r3(line["roofline"].get("fp64_pipe_frac")),
                       "e2e_mlups": r3((line.get("e2e") or {}).get("value"))}}
     for name, f in (line.get("forms") or {}).items():
         s[f"{name}_8192"] = {"mlups": r3(f["value"]), "hbm_frac": r3(f["roofline"]["frac"])}
@@ -787,8 +779,6 @@ def run_ours(args):
     peaks, src = _peaks()
     hbm_peak = float(peaks["hbm_gbs"])
     gbs = BYTES_PER_CCU_F64 * cells / per_launch / 1e9
-    sm_mhz = clocks.get("sm_mhz") or 2070.0
-    fp64_peak = SMS * DFMA_PER_CLK_PER_SM * 2 * sm_mhz * 1e6 / 1e12
     if args.precision != "f64":
         bpn = FORMS[args.precision][1]
         gb = bpn * cells / per_launch / 1e9
@@ -797,17 +787,12 @@ def run_ours(args):
                 "traffic": tr * cells if tr else None, "kernel": f"k_step2<{args.precision}>",
                 "bytes_per_ccu": bpn, "peak_source": f"{src} hbm_gbs"}
     else:
-        ach = FP64_FLOP_PER_CCU * cells / per_launch / 1e12
-        inst_rate = FP64_INST_PER_CCU * cells / per_launch
-        inst_peak = SMS * DFMA_PER_CLK_PER_SM * sm_mhz * 1e6
-        roof = {"bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "TFLOP/s", "frac": ach / fp64_peak,
+        # FP64 values; exact fixed-point sums and FP32 pairs on the integer and FP32
+        # pipes (an FP64 instruction holds its pipe for 64 cycles per warp)
+        roof = {"bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
                 "traffic": DRAM_BYTES_PER_CCU_MEASURED * cells,
-                "kernel": "k_step<StoreF64, shift, forchheimer>", "flop_per_ccu": FP64_FLOP_PER_CCU,
-                "peak_source": f"FP64 pipe: {SMS} SMs x {DFMA_PER_CLK_PER_SM} DFMA/clk x 2 flop x {sm_mhz:.0f} MHz "
-                               "(median SM clock, timed region)",
-                "fp64_pipe_frac": inst_rate / inst_peak,
-                "hbm": {"achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
-                        "bytes_per_ccu": BYTES_PER_CCU_F64, "peak_source": f"{src} hbm_gbs"}}
+                "kernel": "k_step_f64<shift, forchheimer>", "bytes_per_ccu": BYTES_PER_CCU_F64,
+                "peak_source": f"{src} hbm_gbs"}
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t / args.steps * 1e3, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,

@@ -15,7 +15,9 @@
  * BF16 tensor cores with FP32 accumulation, on tcgen05 (accumulator in
  * TMEM): fed by TMA copies when the pixels tile into whole image rows and
  * the channel counts are multiples of 8 (for the forward pass: when the
- * transposed weights are given), otherwise from operands gathered through
+ * transposed weights are given; 3x3 weight gradients with channels in multiples
+ * of 32, and 3x3 layers of 32 gathered channels on rows of a multiple of 128, keep
+ * image rows in a ring and fetch each once), otherwise from operands gathered through
  * registers when the gathered channel count is a multiple of 8 and the
  * operands are 16-byte aligned; the 1x1 convolution to 4 outputs runs on
  * CUDA cores; other shapes on an mma.sync implicit GEMM.  A TMA box that

@@ -21,11 +21,11 @@
 // straight to Eq. 32, so they are never formed.
 //
 // Two storage forms share this arithmetic (templated on the real type R):
-//   StoreF64 : FP64 distributions, FP64 arithmetic, per-node FP64 constants
-//              (1/phi, phi/2, phi nu/K, l1 or 1/(2 l0)) precomputed at init.
-//              On GB300 FP64 issues at 2 DFMA/clk/SM, so this form is bound
-//              by FP64 instruction throughput, not by HBM; precomputing the
-//              constants removes their divisions and square roots.
+//   StoreF64 : FP64 distributions, per-node constants precomputed at init.
+//              On GB300 an FP64 instruction holds its pipe for 64 cycles per
+//              warp, so the step (k_step_f64) computes in fixed point and pairs
+//              of FP32 (clb_split.cuh); the FP64 arithmetic below serves values
+//              outside their range and the reductions.  Bound by issue.
 //   StoreH16 : FP16 storage of each distribution's deviation from its
 //              rest-state value (w_i rho_0 for f, the equilibrium at T0 for
 //              g), FP32 arithmetic, constants recomputed per node from an
