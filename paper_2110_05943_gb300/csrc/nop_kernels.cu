@@ -904,17 +904,18 @@ __global__ void __launch_bounds__(TM_THREADS, 2) k_conv_tma(const __grid_constan
 }
 
 // ---------------------------------------------------------------- row-ring convolution
-// Forward and input gradient of 3x3 layers with 32 (padded) input channels on
-// images whose width is a multiple of 128: k_conv_tma fetches every pixel once per tap (nine boxes per 128-pixel
-// tile), and those copies' request rate, not the MMAs, set its pace.  Here a
-// CTA walks down the image: each 128-pixel row segment is fetched once, with
-// one pixel of halo on either side, into a ring of `stages`; the tile of row y
+// Forward and input gradient of 3x3 layers with 32, 64 or 96 gathered channels
+// (NCH chunks of 32) on images whose width is a multiple of 128: k_conv_tma fetches
+// every pixel once per tap (nine boxes per 128-pixel tile), and those copies'
+// request rate, not the MMAs, set its pace.  Here a CTA walks down the image: each
+// 128-pixel row segment is fetched once, with one pixel of halo on either side,
+// into a ring of `stages`; the tile of row y
 // takes its nine taps from the three newest rows.  A tap's dx only moves the
 // start of the K-major operand by one pixel's bytes (the swizzle follows the
 // address).  All weights stay in shared memory.  Same products in the same
 // order as k_conv_tma (taps, then channels): the same bits.  Roles, TMEM
 // double buffering and bounded waits as there.
-template <int MODE>
+template <int MODE, int NCH>
 __global__ void __launch_bounds__(TM_THREADS, 2)
     k_conv_row(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                const float* __restrict__ bias, const __nv_bfloat16* __restrict__ mask, void* __restrict__ out, int out_f32,
@@ -923,8 +924,8 @@ __global__ void __launch_bounds__(TM_THREADS, 2)
     unsigned char* const wsm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // weights, then the ring
     __shared__ __align__(16) float s_bias[TM_BIAS_MAX];
     constexpr int kc = 32, rb = kc * 2;                                  // channels, and bytes per pixel
-    const int b_bytes = tile_n * kc * 2, stage_bytes = a_bytes;
-    unsigned char* const smem = wsm + 9 * b_bytes;
+    const int b_bytes = tile_n * kc * 2, stage_bytes = NCH * a_bytes;
+    unsigned char* const smem = wsm + 9 * NCH * b_bytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + stages * stage_bytes);
     uint64_t* empty = full + stages;
     uint64_t* acc_full = empty + stages;                                 // [2]
@@ -977,11 +978,12 @@ __global__ void __launch_bounds__(TM_THREADS, 2)
     if (warp == 8) {
         if (lane == 0) {   // producer
             const uint32_t wb = smem_u32(wfull);
-            mbar_expect_tx(wb, (uint32_t)(9 * b_bytes));
-            for (int tap = 0; tap < 9; ++tap) {
-                const uint32_t dst = smem_u32(wsm) + (uint32_t)(tap * b_bytes);
-                if (MODE == FWD) tma_load_3d(dst, &mapB, wb, 0, tap, 0);
-                else tma_load_3d(dst, &mapB, wb, 0, 0, tap);
+            mbar_expect_tx(wb, (uint32_t)(9 * NCH * b_bytes));
+            for (int q = 0; q < 9 * NCH; ++q) {
+                const uint32_t dst = smem_u32(wsm) + (uint32_t)(q * b_bytes);
+                const int tap = q / NCH, c0 = (q % NCH) * kc;
+                if (MODE == FWD) tma_load_3d(dst, &mapB, wb, c0, tap, 0);
+                else tma_load_3d(dst, &mapB, wb, c0, 0, tap);
             }
             int it = 0, st = 0, ph = 0;
             for (int t = t0; t < t1 && ok;) {
@@ -993,8 +995,8 @@ __global__ void __launch_bounds__(TM_THREADS, 2)
                         break;
                     }
                     const uint32_t fb = smem_u32(&full[st]), base = smem_u32(smem + st * stage_bytes);
-                    mbar_expect_tx(fb, (uint32_t)((TC_M + 2) * rb));
-                    tma_load_4d(base, &mapA, fb, 0, w0 - 1, x, img);
+                    mbar_expect_tx(fb, (uint32_t)(NCH * (TC_M + 2) * rb));
+                    for (int c = 0; c < NCH; ++c) tma_load_4d(base + c * a_bytes, &mapA, fb, c * kc, w0 - 1, x, img);
                     ++it;
                     if (++st == stages) {
                         st = 0;
@@ -1036,9 +1038,14 @@ __global__ void __launch_bounds__(TM_THREADS, 2)
                             const int ddy = MODE == FWD ? tap / 3 - 1 : 1 - tap / 3, ddx = MODE == FWD ? tap % 3 - 1 : 1 - tap % 3;
                             const uint32_t al = lo[ddy + 1] + (uint32_t)((1 + ddx) * rb / 16);
 #pragma unroll
-                            for (int ks = 0; ks < kc / 16; ++ks)
-                                tc_mma_lo(d, al + 2 * ks, desc_hi(rb), bl + 2 * ks, desc_hi(rb), idesc, (tap > 0 || ks > 0) ? 1u : 0u);
-                            bl += (uint32_t)(b_bytes >> 4);
+                            for (int c = 0; c < NCH; ++c) {
+                                const uint32_t ac = al + (uint32_t)(c * (a_bytes >> 4));
+#pragma unroll
+                                for (int ks = 0; ks < kc / 16; ++ks)
+                                    tc_mma_lo(d, ac + 2 * ks, desc_hi(rb), bl + 2 * ks, desc_hi(rb), idesc,
+                                              (tap > 0 || c > 0 || ks > 0) ? 1u : 0u);
+                                bl += (uint32_t)(b_bytes >> 4);
+                            }
                         }
                         tc_commit(smem_u32(&empty[p2]));
                         if (x == yb) {
@@ -1800,8 +1807,8 @@ bool launch_tma(const void* A, const void* B, const float* bias, const void* mas
 }
 
 // Launches the row-ring kernel; false when the shape is not one it takes: 3x3,
-// width a multiple of 128, 32 input channels, at most 256 outputs (a multiple of
-// 16).  Measured at 16 x 128^2 against k_conv_tma (both with the present epilogue
+// width a multiple of 128, 32, 64 or 96 input channels, at most 256 outputs (a
+// multiple of 16) whose weights fit in shared memory.  Measured at 16 x 128^2 against k_conv_tma (both with the present epilogue
 // and issue loops): 32 -> 32 20.9 us against 25.0, 32 -> 96 41 against 51; with
 // more input channels it is no faster (96 -> 32: 47.5 against 46.3) or slower
 // (3 x 128^2, 64 -> 64: 14.7 against 12.5: one CTA per SM), so those stay there.
@@ -1809,15 +1816,21 @@ template <int MODE>
 bool launch_row(const void* A, const void* B, const float* bias, const void* mask, void* out, int out_f32, int relu,
                 ConvShape s, long long M, long long N, cudaStream_t st, int* rc) {
     const int C = MODE == FWD ? s.cin : s.cout;
-    if (s.taps != 9 || s.w % TC_M || C != 32 || N % 16 || N > 256 || !aligned16(A) || !aligned16(B)) return false;
+    if (s.taps != 9 || s.w % TC_M || (C != 32 && C != 64 && C != 96) || N % 16 || N > 256 || !aligned16(A) || !aligned16(B)) return false;
+    // 64 channels leave one CTA per SM and pay with several tiles in each and 64
+    // outputs or more (16 x 128^2, us, k_conv_tma / here: 64 -> 64 29.1 / 24.7, its
+    // input gradient 34 / 27.7, 64 -> 96 34.8 / 26.6, but 64 -> 32 22.6 / 23.7; one
+    // image, 64 -> 96: 6.6 / 6.9); 96 always do (96 -> 32 44.1 / 31.6, one image 8.4 / 6.4)
+    if (C == 64 && (N < 64 || M / TC_M < 2LL * sm_count())) return false;
     const long long cmax = s.cin > s.cout ? s.cin : s.cout;
     if (M * cmax * s.taps >= 2147483647LL || M * N >= 2147483647LL) return false;
     const int tile_n = (int)N;
     int cols = 32;
     while (cols < tile_n) cols <<= 1;
     constexpr int kc = 32;
+    const int nch = C / kc;
     const int a_bytes = ((TC_M + 2) * kc * 2 + 1023) / 1024 * 1024;
-    const size_t w_bytes = (size_t)9 * tile_n * kc * 2, stage_bytes = (size_t)a_bytes;
+    const size_t w_bytes = (size_t)9 * tile_n * C * 2, stage_bytes = (size_t)nch * a_bytes;
     // two CTAs per SM where TMEM and shared memory hold them (see launch_tma)
     int per_sm = 2 * cols <= 256 ? 2 : 1;
     long long stages = 0;
@@ -1847,14 +1860,15 @@ bool launch_row(const void* A, const void* B, const float* bias, const void* mas
         if (!encode_map(&mb, B, 3, dims, strides, box, sw)) return false;
     }
     const size_t smem = 1024 + w_bytes + stages * stage_bytes + (2 * stages + 6) * 8 + 16;
-    if (cudaFuncSetAttribute(k_conv_row<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    const auto kern = nch == 1 ? k_conv_row<MODE, 1> : nch == 2 ? k_conv_row<MODE, 2> : k_conv_row<MODE, 3>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         *rc = CLB_NOP_ERR_CUDA;
         return true;
     }
     const long long total = M / TC_M;
     const unsigned grid = (unsigned)std::min<long long>(total, (long long)sm_count() * per_sm);
     const int vec_out = N % 8 == 0 && aligned16(out) && (!mask || aligned16(mask));
-    launch_pdl(k_conv_row<MODE>, dim3(grid), TM_THREADS, smem, st, ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu,
+    launch_pdl(kern, dim3(grid), TM_THREADS, smem, st, ma, mb, bias, (const __nv_bfloat16*)mask, out, out_f32, relu,
                s, (int)N, tile_n, cols, vec_out, (int)stages, a_bytes, (int)total);
     *rc = cudaGetLastError() == cudaSuccess ? CLB_NOP_OK : CLB_NOP_ERR_CUDA;
     return true;
