@@ -527,8 +527,8 @@ extern "C" int clb_batch_set_active(clb_batch* b, const int32_t* active) {
 }
 
 template <class P>
-static void batch_nusselt_as(clb_batch* b, int side) {
-    k_nusselt_batch<P><<<(unsigned)b->cases.size(), kRedThreads, 0, b->stream>>>(
+static void batch_nusselt_as(clb_batch* b, int side, size_t ncase) {
+    k_nusselt_batch<P><<<(unsigned)ncase, kRedThreads, 0, b->stream>>>(
         (const CaseT<typename P::R, typename P::S>*)b->table, b->cur, b->geom, side, b->nu);
 }
 
@@ -539,7 +539,10 @@ extern "C" int clb_batch_nusselt(clb_batch* b, int32_t side, double* nu) {
     batch_sync_cases(b);
     if (side < 0 || side > 3) return bfail(b, CLB_ERR_ARG, "clb_batch_nusselt: case 0: clb_nusselt: side must be 0..3");
     const size_t nc = b->cases.size();
-    size_t bad = nc;   // the first case whose grid has no such number; the cases before it are still given
+    // The first case whose grid has no such number.  The cases before it are
+    // still given; it and those after it are not launched (a grid of one or two
+    // nodes, periodic across the wall, has no third node to read).
+    size_t bad = nc;
     for (size_t c = 0; c < nc; ++c) {
         const clb_params& p = b->cases[c]->prm;
         b->cur_host[c] = b->cases[c]->par;
@@ -547,11 +550,11 @@ extern "C" int clb_batch_nusselt(clb_batch* b, int32_t side, double* nu) {
     }
     if (bad > 0) {
         CKB(b, cudaMemcpyAsync(b->cur, b->cur_host, nc * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-        if (b->prec == CLB_F16S) batch_nusselt_as<StoreH16>(b, side);
-        else if (b->prec == CLB_F16N) batch_nusselt_as<StoreH16N>(b, side);
-        else batch_nusselt_as<StoreF64>(b, side);
+        if (b->prec == CLB_F16S) batch_nusselt_as<StoreH16>(b, side, bad);
+        else if (b->prec == CLB_F16N) batch_nusselt_as<StoreH16N>(b, side, bad);
+        else batch_nusselt_as<StoreF64>(b, side, bad);
         CKB(b, cudaGetLastError());
-        CKB(b, cudaMemcpyAsync(b->nu_host, b->nu, nc * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+        CKB(b, cudaMemcpyAsync(b->nu_host, b->nu, bad * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
         CKB(b, cudaStreamSynchronize(b->stream));
     }
     for (size_t c = 0; c < bad; ++c) {

@@ -93,7 +93,8 @@ __global__ void __launch_bounds__(kRedThreads) k_nusselt_partial(const BufT<type
     if (threadIdx.x == 0) partial[blockIdx.x] = v;
 }
 
-// Nusselt numbers of one wall of every case of a batch, a block per case:
+// Nusselt numbers of one wall of the cases of a batch, a block per case (each
+// with two nodes along the wall and three across it at least):
 // one launch and one copy for the whole batch (512 cases: 27 ms with two
 // launches, a copy and a wait each, 0.1 ms now).  cur[c]: the case's current
 // buffer; geom[c] = (L, dT).  The sums of 256 nodes and the sum over them run
