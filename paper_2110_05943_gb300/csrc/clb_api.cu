@@ -48,6 +48,7 @@ struct clb_handle {
     KParamsT<float> k32{};        // FP16 forms
     SplitPhys sp{};               // FP64 form: the constants of its split arithmetic
     int prec = CLB_F64;
+    int sms = 1;                  // streaming multiprocessors of the device
     size_t es = 8;                // bytes per stored distribution value
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
@@ -74,6 +75,7 @@ struct clb_handle {
     bool graph_failed = false;
     dim3 block, grid;          // one node per thread
     dim3 block2, grid2;        // two nodes per thread (FP16 forms)
+    bool overlap = false, edge_last = false;   // see pick_launch
     // FP16N form: tensor maps of the TMA-fed interior (per input buffer: f
     // planes, g planes, records; and 1/phi), its tiling, and the wait bound
     CUtensorMap tm_f[2], tm_g[2], tm_r[2], tm_i;
@@ -84,8 +86,8 @@ struct clb_handle {
 
     AuxT<double> aux64() const { return AuxT<double>{coef, nullptr, nullptr, (const double*)ayg, scoef}; }
     AuxT<float> aux32() const {
-        return prec == CLB_F16N ? AuxT<float>{nullptr, nullptr, phi32, (const float*)ayg, nullptr}
-                                : AuxT<float>{nullptr, phi32, nullptr, (const float*)ayg, nullptr};
+        return prec == CLB_F16N ? AuxT<float>{nullptr, nullptr, phi32, (const float*)ayg}
+                                : AuxT<float>{nullptr, phi32, nullptr, (const float*)ayg};
     }
     template <typename S>
     BufT<S> buf(int i) const { return BufT<S>{(S*)f[i], (S*)g[i], rec[i], seq ? seq + i : nullptr}; }
@@ -231,6 +233,23 @@ static void pick_launch(clb_handle* h) {
     const int nx = h->prm.nx, ny = h->prm.ny;
     shape_blocks(nx, ny, CLB_F64_BX, CLB_F64_THREADS, h->block, h->grid);
     shape_blocks((nx + 1) / 2, ny, CLB_F16_BX, 128, h->block2, h->grid2);
+    // How the FP16 steps are launched, by the number of rounds their blocks take
+    // (room: those resident at once by the launch bounds).
+    // Steps overlap (pdl_begin) from 2.1 rounds on: F16S 1531 x 389 8.3 us against 8.7
+    // one after the other, 1024^2 13.9 and 14.2, 4096^2 211.4 and 216.  In a grid of
+    // about one round the next steps' waiting blocks sit where this one's should go,
+    // and it spreads unevenly: F16S 512^2 18 us against 7, 64 x 2048 10.1 against 5.9,
+    // F16N 48 x 512 9.1 against 5.4; at two rounds it depends (60 x 8192 16.2 against 13.9,
+    // 700^2 periodic 9.6 and 8.1, 700^2 cavity 7.8 and 8.1).
+    // An F16S step that does not overlap keeps the read-only loads:
+    // 256^2 4.5 us, 4.8 with the coherent ones (F16N 128^2: 5.9 and 5.4, so it does not).
+    // The edge blocks of F16S come last up to 1.25 rounds: see k_step2.
+    const bool s16 = h->prec == CLB_F16S;
+    const long long room = (long long)h->sms * (s16 ? Step2MinBlocks<StoreH16>::value : Step2MinBlocks<StoreH16N>::value);
+    const long long threads = h->block2.x * h->block2.y;
+    const long long nb = (long long)h->grid2.x * h->grid2.y + (edge_count(h->k32.g) + threads - 1) / threads;
+    h->overlap = 10 * nb >= 21 * room;
+    h->edge_last = s16 && 4 * nb < 5 * room;
 }
 
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime
@@ -325,10 +344,10 @@ static void free_all(clb_handle* h) {
 }
 
 // ------------------------------------------------------------------ kernels
-// Launch that may start before the kernel in front of it has ended; the
-// kernel itself waits for it (pdl_begin).
+// Launch of a kernel that begins with pdl_begin; with `overlap` it may start
+// before the kernel in front of it has ended, and waits for it there.
 template <class... P, class... V>
-static void launch_pdl(void (*k)(P...), unsigned grid, dim3 block, cudaStream_t s, const V&... v) {
+static void launch_step_kernel(bool overlap, void (*k)(P...), unsigned grid, dim3 block, cudaStream_t s, const V&... v) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = block;
@@ -337,8 +356,12 @@ static void launch_pdl(void (*k)(P...), unsigned grid, dim3 block, cudaStream_t 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     cudaLaunchKernelEx(&cfg, k, P(v)...);   // an error stays for the caller's cudaGetLastError
+}
+template <class... P, class... V>
+static void launch_pdl(void (*k)(P...), unsigned grid, dim3 block, cudaStream_t s, const V&... v) {
+    launch_step_kernel(true, k, grid, block, s, v...);
 }
 
 static void step_f64(clb_handle* h, cudaStream_t s) {
@@ -361,9 +384,8 @@ template <class P>
 static void step2_as(clb_handle* h, cudaStream_t s, long long limit = TT_LIMIT, int selftest = 0) {
     using S = typename P::S;
     const BufT<S> in = h->buf<S>(h->par), out = h->buf<S>(1 - h->par);
-    const AuxT<float> A = h->aux32();
     const bool sh = h->prm.shift != 0, fo = h->prm.forchheimer != 0;
-    // pair tiles (interior pairs only), then the edge nodes (see k_step2);
+    // pair tiles (interior pairs only) and the edge nodes (see k_step2);
     // with the TMA-fed interior, the pair tiles cover only the rows 0 and
     // ny - 1 of a periodic y
     const Geo& G = h->k32.g;
@@ -374,16 +396,16 @@ static void step2_as(clb_handle* h, cudaStream_t s, long long limit = TT_LIMIT, 
             const int b = h->par;
             const dim3 gr((unsigned)h->tma_grid), bl(TT_THREADS);
             if (sh && fo)
-                k_step2n_tma<true, true><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, A,
+                k_step2n_tma<true, true><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, h->aux32(),
                                                                  h->k32, h->tma_tiles_x, h->tma_ntiles, limit, selftest, h->tma_fail);
             else if (sh)
-                k_step2n_tma<true, false><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, A,
+                k_step2n_tma<true, false><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, h->aux32(),
                                                                   h->k32, h->tma_tiles_x, h->tma_ntiles, limit, selftest, h->tma_fail);
             else if (fo)
-                k_step2n_tma<false, true><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, A,
+                k_step2n_tma<false, true><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, h->aux32(),
                                                                   h->k32, h->tma_tiles_x, h->tma_ntiles, limit, selftest, h->tma_fail);
             else
-                k_step2n_tma<false, false><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, A,
+                k_step2n_tma<false, false><<<gr, bl, TT_SMEM, s>>>(h->tm_f[b], h->tm_g[b], h->tm_r[b], h->tm_i, in, out, h->aux32(),
                                                                    h->k32, h->tma_tiles_x, h->tma_ntiles, limit, selftest, h->tma_fail);
             nt = G.wall_y ? 0 : tx;
             outer = 1;
@@ -392,23 +414,37 @@ static void step2_as(clb_handle* h, cudaStream_t s, long long limit = TT_LIMIT, 
     const int threads = (int)(h->block2.x * h->block2.y);
     const unsigned nb = (unsigned)(nt + (edge_count(G) + threads - 1) / threads);
     if (nb == 0) return;
-    if (outer) {
-        if (sh && fo) launch_pdl(k_step2<P, true, true, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
-        else if (sh) launch_pdl(k_step2<P, true, false, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
-        else if (fo) launch_pdl(k_step2<P, false, true, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
-        else launch_pdl(k_step2<P, false, false, true>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
-    } else {
-        if (sh && fo) launch_pdl(k_step2<P, true, true, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
-        else if (sh) launch_pdl(k_step2<P, true, false, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
-        else if (fo) launch_pdl(k_step2<P, false, true, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
-        else launch_pdl(k_step2<P, false, false, false>, nb, h->block2, s, in, out, A, h->k32, tx, nt);
+    typename Step2Aux<P>::type A{};
+    static_cast<AuxT<float>&>(A) = h->aux32();
+    auto go = [&](auto kernel) { launch_step_kernel(h->overlap && !outer, kernel, nb, h->block2, s, in, out, A, h->k32, tx, nt); };
+    if constexpr (std::is_same<P, StoreH16NT<LdPD>>::value) {
+        if (outer) {
+            if (sh && fo) go(k_step2<P, true, true, true>);
+            else if (sh) go(k_step2<P, true, false, true>);
+            else if (fo) go(k_step2<P, false, true, true>);
+            else go(k_step2<P, false, false, true>);
+            return;
+        }
     }
+    if constexpr (std::is_same<P, StoreH16>::value) {
+        if (h->edge_last) {
+            if (sh && fo) go(k_step2<P, true, true, false, true>);
+            else if (sh) go(k_step2<P, true, false, false, true>);
+            else if (fo) go(k_step2<P, false, true, false, true>);
+            else go(k_step2<P, false, false, false, true>);
+            return;
+        }
+    }
+    if (sh && fo) go(k_step2<P, true, true>);
+    else if (sh) go(k_step2<P, true, false>);
+    else if (fo) go(k_step2<P, false, true>);
+    else go(k_step2<P, false, false>);
 }
 
 static void launch_step(clb_handle* h, cudaStream_t s) {
-    if (h->prec == CLB_F16S) step2_as<StoreH16T<LdPD>>(h, s);
+    if (h->prec == CLB_F64) step_f64(h, s);
     else if (h->prec == CLB_F16N) step2_as<StoreH16NT<LdPD>>(h, s);
-    else step_f64(h, s);
+    else h->overlap ? step2_as<StoreH16T<LdPD>>(h, s) : step2_as<StoreH16>(h, s);
     h->par = 1 - h->par;
 }
 
@@ -518,6 +554,7 @@ extern "C" int clb_init(clb_handle** out, const clb_params* p, const double* phi
         }                                                                                         \
     } while (0)
     CKI(cudaGetDevice(&h->device));
+    CKI(cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device));
     CKI(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
 
     h->prec = p->precision;

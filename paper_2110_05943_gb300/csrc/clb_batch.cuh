@@ -193,10 +193,11 @@ static void batch_launch_as(clb_batch* b, cudaStream_t s, cudaStream_t side) {
             const unsigned g = (unsigned)b->n_work;
             const int4 *w = b->work, *t = b->itiles, *e = b->echunks;
             const int n = b->n_itiles, pc = b->per_cta, par = b->par;
-            if (b->shift && b->forch) launch_pdl(k_step_batch_mix<P, true, true>, g, block, s, tab, w, t, n, pc, e, par);
-            else if (b->shift) launch_pdl(k_step_batch_mix<P, true, false>, g, block, s, tab, w, t, n, pc, e, par);
-            else if (b->forch) launch_pdl(k_step_batch_mix<P, false, true>, g, block, s, tab, w, t, n, pc, e, par);
-            else launch_pdl(k_step_batch_mix<P, false, false>, g, block, s, tab, w, t, n, pc, e, par);
+            constexpr bool pdl = std::is_same<typename P::Ld, LdPD>::value;
+            if (b->shift && b->forch) launch_step_kernel(pdl, k_step_batch_mix<P, true, true>, g, block, s, tab, w, t, n, pc, e, par);
+            else if (b->shift) launch_step_kernel(pdl, k_step_batch_mix<P, true, false>, g, block, s, tab, w, t, n, pc, e, par);
+            else if (b->forch) launch_step_kernel(pdl, k_step_batch_mix<P, false, true>, g, block, s, tab, w, t, n, pc, e, par);
+            else launch_step_kernel(pdl, k_step_batch_mix<P, false, false>, g, block, s, tab, w, t, n, pc, e, par);
             return;
         }
         const bool fork = side && b->n_itiles > 0 && b->n_echunks > 0;
@@ -283,9 +284,14 @@ static cudaError_t batch_persist(clb_batch* b, cudaStream_t s, int par0, int nst
 
 static void batch_launch(clb_batch* b, cudaStream_t s, cudaStream_t side = nullptr) {
     if (b->ntiles > 0) {
-        if (b->prec == CLB_F16S) batch_launch_as<StoreH16T<LdPD>, 2>(b, s, side);
-        else if (b->prec == CLB_F16N) batch_launch_as<StoreH16NT<LdPD>, 2>(b, s, side);
-        else batch_launch_as<StoreF64T<LdPD>, 1>(b, s, side);
+        // FP16 steps overlap from three rounds of resident blocks on (see pick_launch; a
+        // block takes several tiles here, so two rounds spread less evenly): 24 cases of 64 to 200 nodes a side, F16N, 17.9 us a step one after the
+        // other, 24.5 overlapping; 512 of up to 1024: 1.28 ms overlapping
+        const bool overlap = b->n_work >= 3LL * b->cases[0]->sms * CLB_BATCH_MIX_MINB;
+        if (b->prec == CLB_F64) batch_launch_as<StoreF64T<LdPD>, 1>(b, s, side);
+        else if (b->prec == CLB_F16S)
+            overlap ? batch_launch_as<StoreH16T<LdPD>, 2>(b, s, side) : batch_launch_as<StoreH16, 2>(b, s, side);
+        else overlap ? batch_launch_as<StoreH16NT<LdPD>, 2>(b, s, side) : batch_launch_as<StoreH16N, 2>(b, s, side);
     }
     b->par = 1 - b->par;
 }

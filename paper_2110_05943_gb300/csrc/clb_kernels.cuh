@@ -45,6 +45,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "clb_split.cuh"
 
 #ifndef CLB_HD
@@ -116,7 +118,14 @@ struct AuxT {
     const float* phi;
     const float* ip;
     const R* ayg;
-    const float2* scoef;   // FP64 form: the constants as split numbers, kSplitPlanes dense planes
+};
+template <>
+struct AuxT<double> {
+    const CoefT<double>* coef;
+    const float* phi;
+    const float* ip;
+    const double* ayg;
+    const float2* scoef;   // the constants as split numbers, kSplitPlanes dense planes
 };
 
 // One ping-pong buffer: distribution planes, and for the equilibrium-shifted
@@ -1586,13 +1595,15 @@ __host__ __device__ __forceinline__ void edge_node(const Geo& G, long long i, in
 }
 
 // One launch, two kinds of blocks (no warp mixes the packed and the
-// per-node path): the last n_tiles blocks cover all pairs of the grid in
+// per-node path): n_tiles blocks cover all pairs of the grid in
 // tiles_x x ... tiles of blockDim pairs, aligned at x = 0 so that a warp's
 // 64 nodes are one 128-byte line of every FP16 plane, and skip the pairs
-// that are not interior; the blocks before them take the edge nodes, one per
-// thread.  The edge blocks start first: one takes several times as long as a
-// tile, and at the end of the grid they ran on alone (F16S channel 1531 x 389
-// 11.1 us a step against 8.8 now, F16N 512^2 12.0 against 8.8).
+// that are not interior; the others take the edge nodes, one per thread.  Edge
+// blocks take several times as long as a tile and come first: at the end of the
+// grid they run on alone (F16S channel 1531 x 389 11.3 us a step with them last,
+// 8.8 first; F16N 512^2 11.9 and 8.6).  LAST: after the tiles, for F16S grids whose
+// blocks are all resident at once (64 x 2048 channel 6.4 us first, 5.9 last; 256 x
+// 1024 7.2 and 6.9).
 // Resident 128-thread blocks per SM the registers of k_step2 are capped
 // for, per form (measured at 8192^2 with 64 x 2-thread blocks): the
 // rest-shifted form runs 7 (72 registers, 48 bytes of spills, 28 warps:
@@ -1613,17 +1624,34 @@ struct Step2MinBlocks<StoreH16T<L>> {
     static constexpr int value = CLB_F16S_MINB;
 };
 
+// k_step2's auxiliary pointers.  The overlapping F16S kernel gets eight bytes
+// more, which move the constants behind them off a 16-byte boundary: the compiler
+// then schedules the same arithmetic better for a full chip (4096^2 211.4 us a
+// step against 216.3), the other way round for a chip that one round of blocks fills
+// (64 x 2048 channel 5.9 us without, 6.3 with).
+struct AuxPad : AuxT<float> {
+    const void* pad;
+};
+template <class P>
+struct Step2Aux {
+    using type = AuxT<float>;
+};
+template <>
+struct Step2Aux<StoreH16T<LdPD>> {
+    using type = AuxPad;
+};
+
 // OUTER: the pair tiles cover only the rows 0 and ny - 1 (thread rows 0 and
 // 1 of one band of tiles), the other rows' interior pairs being taken by the
 // TMA-fed kernel.
-template <class P, bool SHIFT, bool FORCH, bool OUTER = false>
+template <class P, bool SHIFT, bool FORCH, bool OUTER = false, bool LAST = false>
 __global__ void __launch_bounds__(128, Step2MinBlocks<P>::value)
     k_step2(const BufT<typename P::S> in, const BufT<typename P::S> out,
-                                                  const AuxT<float> A, const KParamsT<float> K, int tiles_x,
+                                                  const typename Step2Aux<P>::type A, const KParamsT<float> K, int tiles_x,
                                                   int n_tiles) {
-    pdl_begin();
-    const int n_edge = (int)gridDim.x - n_tiles, b = (int)blockIdx.x - n_edge;
-    if (b >= 0) {
+    if constexpr (std::is_same<typename P::Ld, LdPD>::value) pdl_begin();
+    const int b = (int)blockIdx.x - (LAST ? 0 : (int)gridDim.x - n_tiles);
+    if (LAST ? b < n_tiles : b >= 0) {
         const int x0 = 2 * ((b % tiles_x) * blockDim.x + threadIdx.x);
         int y = (b / tiles_x) * blockDim.y + threadIdx.y;
         if constexpr (OUTER) {
@@ -1636,7 +1664,8 @@ __global__ void __launch_bounds__(128, Step2MinBlocks<P>::value)
         if (y >= K.g.ny || !interior_pair(K.g, x0, y)) return;
         step_pair_interior<P, SHIFT, FORCH>(in, out, A, K, x0, y);
     } else {
-        const long long i = (long long)blockIdx.x * (blockDim.x * blockDim.y) + threadIdx.y * blockDim.x + threadIdx.x;
+        const long long i = (long long)(LAST ? b - n_tiles : (int)blockIdx.x) * (blockDim.x * blockDim.y) +
+                            threadIdx.y * blockDim.x + threadIdx.x;
         if (i >= edge_count(K.g)) return;
         int x, y;
         edge_node(K.g, i, x, y);
@@ -1820,7 +1849,7 @@ __global__ void __launch_bounds__(128, CLB_BATCH_MIX_MINB)
                      const int4* __restrict__ tiles, int ntiles, int per_cta, const int4* __restrict__ chunks, int par) {
     __shared__ __align__(16) unsigned char raw[sizeof(CaseT<typename P::R, typename P::S>)];
     const int4 w = __ldg(work + blockIdx.x);
-    pdl_begin();
+    if constexpr (std::is_same<typename P::Ld, LdPD>::value) pdl_begin();
     if (w.x == 0) batch_int_tiles<P, SHIFT, FORCH>(cases, tiles, w.y, min(w.y + per_cta, ntiles), par, raw);
     else batch_edge_chunk<P, SHIFT, FORCH>(cases, __ldg(chunks + w.y), par, raw);
 }
