@@ -50,9 +50,10 @@ enum { CLB_PERIODIC = 0, CLB_WALL = 1 };
 enum { CLB_ADIABATIC = 0, CLB_ISOTHERMAL = 1 };
 /* Arithmetic / storage form of the distributions (reductions stay FP64).
  *   CLB_F64  : FP64 storage; the step's arithmetic is exact fixed-point sums
- *              and pairs of FP32 (no further from exact arithmetic than FP64
- *              instructions, measured), FP64 instructions where a value leaves
- *              their range; 232 B per node update.
+ *              and pairs of FP32 where these are no further from exact
+ *              arithmetic than FP64 instructions (density within 1/8 of 1,
+ *              speeds below 1/24; any temperature scale), else FP64
+ *              instructions; 232 B per node update.
  *   CLB_F16S : each distribution stored in FP16 as its deviation from the
  *              rest state (w_i rho_0 for f, the D2Q5 equilibrium at u = 0,
  *              T = T0 for g), arithmetic in FP32; 60 B per node update.

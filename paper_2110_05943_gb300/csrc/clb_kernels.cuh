@@ -1389,29 +1389,34 @@ __device__ __forceinline__ SplitCoef split_coef(const AuxT<double>& A, const Geo
     return SplitCoef{v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]};
 }
 
+// The values a node is computed from: f in fixed point (range: see fix_f), g as
+// loaded and the high word of the largest |g| (see split_unit).
 template <class L>
-__device__ __forceinline__ void split_pull(const BufT<double>& in, const Geo& G, const SplitPhys& P, int x, int y,
-                                           long long (&f)[9], long long (&g)[5], uint32_t& range, uint32_t& big) {
+__device__ __forceinline__ void split_pull(const BufT<double>& in, const Geo& G, int x, int y, long long (&f)[9],
+                                           double (&g)[5], uint32_t& range, uint32_t& big) {
     long long o[9];
     sources<long long>(G, x, y, o);
-    double vf[9], vg[5];
+    double vf[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) vf[i] = L::ld(in.f + i * G.plane + o[i]);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) vg[i] = L::ld(in.g + i * G.plane + o[i]);
+    for (int i = 0; i < 5; ++i) g[i] = L::ld(in.g + i * G.plane + o[i]);
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = fix_f(vf[i], range);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) g[i] = fix_g(vg[i], P.gexp, big);
+    for (int i = 0; i < 5; ++i) big = max(big, g_size(g[i]));
 }
 
-__device__ __forceinline__ void split_store(const BufT<double>& out, const Geo& G, const SplitPhys& P, int x, int y,
-                                            const long long (&f)[9], const long long (&g)[5]) {
+__device__ __forceinline__ void split_store_g(const BufT<double>& out, const Geo& G, int gexp, int x, int y,
+                                              const long long (&g)[5]) {
+    const long long o = (long long)y * G.px + x;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) __stwb(out.g + i * G.plane + o, unfix(g[i], 60 - gexp));
+}
+__device__ __forceinline__ void split_store_f(const BufT<double>& out, const Geo& G, int x, int y, const long long (&f)[9]) {
     const long long o = (long long)y * G.px + x;
 #pragma unroll
     for (int i = 0; i < 9; ++i) __stwb(out.f + i * G.plane + o, unfix(f[i]));
-#pragma unroll
-    for (int i = 0; i < 5; ++i) __stwb(out.g + i * G.plane + o, unfix(g[i], 60 - P.gexp));
 }
 
 template <class L, bool SHIFT, bool FORCH>
@@ -1419,12 +1424,31 @@ __device__ __forceinline__ bool split_step_interior(const BufT<double>& in, cons
                                                     const AuxT<double>& A, const Geo& G, const SplitPhys& P, int x,
                                                     int y) {
     long long f[9], g[5];
+    double vg[5];
     uint32_t range = 0u, big = 0u;
     const SplitCoef c = split_coef(A, G, x, y);
-    split_pull<L>(in, G, P, x, y, f, g, range, big);
-    const bool ok = split_node<SHIFT, FORCH>(f, g, c, P);
-    if (!(ok && fix_ok(range) && big < P.gmax)) return false;
-    split_store(out, G, P, x, y, f, g);
+    split_pull<L>(in, G, x, y, f, vg, range, big);
+    const int gexp = split_unit(big, P);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) g[i] = fix_d(vg[i], gexp);
+    SplitMid m;
+    if (!(split_heat<SHIFT, FORCH>(f, g, c, P, gexp, kMaxSpeed, m) && fix_ok(range) && big < P.gmax)) return false;
+    split_store_g(out, G, gexp, x, y, g);
+    if (!split_flow<SHIFT>(f, m, c.ip, P)) return false;
+    split_store_f(out, G, x, y, f);
+    return true;
+}
+
+template <bool SHIFT, bool FORCH, bool REST>
+__device__ __forceinline__ bool split_wall_store(const BufT<double>& out, const Geo& G, const SplitPhys& P, int gexp, int x,
+                                                 int y, const WallInfo& w, long long (&f)[9], long long (&g)[5],
+                                                 long long n0ss, const SplitCoef& cs, const SplitCoef& cb) {
+    SplitMid m;
+    sf Tb;
+    if (!split_wall_heat<SHIFT, FORCH, REST>(f, g, n0ss, cs, w.su, w.st, P, gexp, kMaxSpeed, m, Tb)) return false;
+    split_store_g(out, G, gexp, x, y, g);
+    if (!split_wall_flow<SHIFT, FORCH, REST>(f, m, Tb, cs.ip, cb, w.su, P)) return false;
+    split_store_f(out, G, x, y, f);
     return true;
 }
 
@@ -1433,21 +1457,31 @@ __device__ __forceinline__ bool split_step_wall(const BufT<double>& in, const Bu
                                                 const AuxT<double>& A, const Geo& G, const SplitPhys& P, int x, int y,
                                                 const WallInfo& w) {
     long long f[9], g[5], n0ss = 0;
-    uint32_t range = 0u, big = 0u;
+    double vg[5], vs[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    uint32_t range = 0u, big = w.st < 0 ? 0u : P.wbig[w.st];
     const int sx = x + w.dx, sy = y + w.dy;
     const SplitCoef cs = split_coef(A, G, sx, sy), cb = split_coef(A, G, x, y);
-    split_pull<L>(in, G, P, sx, sy, f, g, range, big);
+    split_pull<L>(in, G, sx, sy, f, vg, range, big);
     if (w.st < 0) {
         long long o[9];
         sources<long long>(G, sx + w.dx, sy + w.dy, o);
 #pragma unroll
-        for (int i = 0; i < 5; ++i) n0ss += fix_g(L::ld(in.g + i * G.plane + o[i]), P.gexp, big);
+        for (int i = 0; i < 5; ++i) {
+            vs[i] = L::ld(in.g + i * G.plane + o[i]);
+            big = max(big, g_size(vs[i]));
+        }
     }
-    const bool ok = P.rest[w.su] ? split_wall<SHIFT, FORCH, true>(f, g, n0ss, cs, cb, w.su, w.st, P)
-                                 : split_wall<SHIFT, FORCH, false>(f, g, n0ss, cs, cb, w.su, w.st, P);
-    if (!(ok && fix_ok(range) && big < P.gmax)) return false;
-    split_store(out, G, P, x, y, f, g);
-    return true;
+    const int gexp = split_unit(big, P);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) g[i] = fix_d(vg[i], gexp);
+    if (w.st < 0) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) n0ss += fix_d(vs[i], gexp);
+    }
+    const bool ok = big < P.gmax && fix_ok(range);
+    return ok && (P.rest[w.su]
+                      ? split_wall_store<SHIFT, FORCH, true>(out, G, P, gexp, x, y, w, f, g, n0ss, cs, cb)
+                      : split_wall_store<SHIFT, FORCH, false>(out, G, P, gexp, x, y, w, f, g, n0ss, cs, cb));
 }
 
 // The FP64 path of a node (out of line: it is rarely taken, and its code and

@@ -10,7 +10,7 @@
 //   * pairs of FP32 values (hi + lo, about 48 bits: "split" numbers) for the
 //     collision's increments, which are small: the state is never held in
 //     less than 60 fractional bits, only the increments' own relative
-//     precision is 2^-46 or so.  The O(1) parts (rho / 3, rho / 9, j / 3,
+//     precision is 2^-46 or so (FP64's: 2^-53).  The O(1) parts (rho / 3, rho / 9, j / 3,
 //     c_sT^2 T) cancel in exact integer arithmetic before anything is
 //     converted, and px = rho u_x - j_x = rho F_x / 2 (the definition of the
 //     implicit velocity, Eqs. 22-23) replaces a difference of large numbers.
@@ -24,14 +24,20 @@
 // for the collision in FP64.  What bounds it now is the sum of the pipes (FMA
 // 61 %, FP64 58 %, integer 44 % busy) at 19 warps per SM.
 //
-// Range.  Fixed point covers rho f_i in [2^-8, 1), |g_i| < 2^gexp (gexp from
-// the run's temperature scale) and increments below 1/16.  A node outside
-// (strong shocks, diverging runs, NaN) takes the FP64 path; nothing is
-// refused that was accepted before.
+// Range.  Fixed point covers f_i in [2^-8, 1); g is carried in a unit of each
+// node's own (split_unit), since fixed point is absolute precision: in the run's unit
+// a temperature of 1e-6 of it kept five digits less than FP64 storage.  A node is left
+// to the FP64 path where the split numbers would be further off than FP64
+// instructions: speeds from 1/24 on (split products of u u have an error of 2^-46
+// u^2), increments of f from 1/64 on, densities more than 1/8 off 1, sigma and
+// varpi whose largest g is below T / 32; and where values leave their range (a
+// g of the run's unit 2^gexp or more, diverging runs, NaN).  Nothing is refused that
+// was accepted before.  T u, which is not small, is a product of fixed-point numbers
+// (split_flux): as a split number it left g up to four times further off.
 //
-// Error against exact arithmetic (checked by tests): the moments' rounding
-// of the FP64 path (5e-17 a step in rho and T) is gone; what the split
-// increments add is smaller.
+// Error against the same formulas in extended precision, one update, over speeds up to
+// the limit, sigma 0.5 to 2, any temperature scale (tests/test_split_precision.py):
+// f 0.2 to 0.5 of the FP64 instructions' in the mean square, g 0.02 to 0.9.
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -67,6 +73,7 @@ CLB_SP long long d2ll(double v) { return __double2ll_rn(v); }
 CLB_SP uint32_t d_hi(double v) { return (uint32_t)__double2hiint(v); }
 CLB_SP uint32_t d_lo(double v) { return (uint32_t)__double2loint(v); }
 CLB_SP double d_make(uint32_t hi, uint32_t lo) { return __hiloint2double((int)hi, (int)lo); }
+CLB_SP float f_make(uint32_t bits) { return __uint_as_float(bits); }
 #else
 // The same on the host (tests and parameter set-up); the estimates are the
 // correctly rounded values there.
@@ -87,6 +94,7 @@ CLB_SP long long d2ll(double v) { return llrint(v); }
 CLB_SP uint32_t d_hi(double v) { uint64_t b; memcpy(&b, &v, 8); return (uint32_t)(b >> 32); }
 CLB_SP uint32_t d_lo(double v) { uint64_t b; memcpy(&b, &v, 8); return (uint32_t)b; }
 CLB_SP double d_make(uint32_t hi, uint32_t lo) { uint64_t b = ((uint64_t)hi << 32) | lo; double v; memcpy(&v, &b, 8); return v; }
+CLB_SP float f_make(uint32_t bits) { float v; memcpy(&v, &bits, 4); return v; }
 #endif
 
 // A split number: the unevaluated sum h + l of two FP32 values.
@@ -170,6 +178,7 @@ CLB_SP sf2 pair(sf a, sf b) { return sf2{float2{a.h, b.h}, float2{a.l, b.l}}; }
 CLB_SP sf2 both(sf a) { return sf2{pboth(a.h), pboth(a.l)}; }
 CLB_SP sf first(sf2 a) { return sf{a.h.x, a.l.x}; }
 CLB_SP sf second(sf2 a) { return sf{a.h.y, a.l.y}; }
+CLB_SP float fmin_f(float a, float b) { return a < b ? a : b; }
 CLB_SP sf2 swp(sf2 a) { return sf2{pswap(a.h), pswap(a.l)}; }
 CLB_SP sf2 neg(sf2 a) { return sf2{pneg(a.h), pneg(a.l)}; }
 CLB_SP sf2 dbl(sf2 a) { return sf2{padd(a.h, a.h), padd(a.l, a.l)}; }
@@ -245,7 +254,18 @@ CLB_SP void to_fix4(sf2 a, long long& x, long long& y) {
     x = (long long)hx * 1073741824LL + (long long)(f2i(m.x) + f2i(l.x));
     y = (long long)hy * 1073741824LL + (long long)(f2i(m.y) + f2i(l.y));
 }
-constexpr float kMaxIncr = 0.0625f;
+constexpr float kMaxIncr = 0.03125f;
+
+// a b / 2^64 for |a|, |b| < 2^63 - 2^31, within two units: three signed 32 x 32
+// products (the low words are rounded into the high ones, so they are signed
+// too); the product of the two low words, less than a unit, is left out.
+CLB_SP long long mul_hi(long long a, long long b) {
+    const uint32_t la = (uint32_t)a, lb = (uint32_t)b;
+    const int ha = (int)((uint32_t)((unsigned long long)a >> 32) + (la >> 31));
+    const int hb = (int)((uint32_t)((unsigned long long)b >> 32) + (lb >> 31));
+    const long long c = (long long)ha * (int)lb + (long long)hb * (int)la;
+    return (long long)ha * hb + (c >> 32);
+}
 
 // FP64 value in [2^-8, 1) to fixed point (exact); x: its high word minus that
 // of 2^-8, in range iff x < 2^23.
@@ -279,20 +299,48 @@ struct SplitPhys {
     sf third, ninth;                 // 1/3, 1/9
     sf sp, sm, sv, s3, s4, s4_3, s4_v, c62;   // s4_3 = s4 - s3, s4_v = s4 - s_v
     sf ca2, c6s, cb8;                // unit shift: 2 (1 - s_v/2), 2 (1 - s3/2), 1 - s4/2
-    sf inv_sigma, hza;               // 1 / sigma, zeta_a / 2
+    sf inv_sigma;                    // 1 / sigma
     double kappa;                    // c_sT^2 / sigma
-    int gexp;                        // temperatures and g are carried in units of 2^gexp
-    float tunit;                     // 2^gexp
-    uint32_t gmax;                   // high word of 2^gexp: |g| stays below it
-    sf uw[4], vw[4], Tw[4];          // walls: velocity, temperature (units of 2^gexp)
-    long long n0w[4], cw[4];         // and sigma T_w, c_sT^2 T_w in fixed point
+    long long sinv;                  // 2^(64 - sshift) / sigma, in [2^60, 2^61]
+    int sshift;
+    long long zeta, om;              // zeta_a, 1 - zeta_a in units of 2^-61
+    int gexp;                        // the coarsest unit 2^gexp of temperatures and g: |g| stays below it
+    int ghead;                       // a node's unit is 2^ghead times the power of two above its largest |g|
+    uint32_t gmax;                   // high word of 2^gexp
+    sf uw[4], vw[4];                 // walls: velocity,
+    long long uwf[4], vwf[4];        // the same in units of 2^-64,
+    double n0w[4], cw[4];            // sigma T_w, c_sT^2 T_w,
+    uint32_t wbig[4];                // and the high word of the largest g at rest (0: adiabatic)
     int rest[4];                     // the wall does not move
 };
 
+// Exponent of the unit in which a node's g and T are carried; big: high word
+// of the largest |g| it is computed from.  Fixed point is absolute precision, so
+// each node takes its own unit, and a temperature small against the run's keeps the
+// digits FP64 storage holds.  (Below 2^-958 the unit stays: FP64's own range ends.)
+CLB_SP int split_unit(uint32_t big, const SplitPhys& P) {
+    const int e = (int)(big >> 20);
+    const int g = (e > 64 ? e : 64) - 1022 + P.ghead;
+    return g < P.gexp ? g : P.gexp;
+}
+// 2^gexp in FP32: temperatures below its range move nothing (the force adds to
+// velocities held to 2^-60).
+CLB_SP float split_tunit(int gexp) { return f_make(gexp > -127 ? (uint32_t)(gexp + 127) << 23 : 0u); }
+// The size of a g: the high word of |g|.
+CLB_SP uint32_t g_size(double v) { return d_hi(v) & 0x7FFFFFFFu; }
+// A double in units of 2^(gexp - 60).
+CLB_SP long long fix_d(double v, int gexp) {
+    uint32_t unused = 0u;
+    return fix_g(v, gexp, unused);
+}
+
 // The constants of a run.  top: the largest temperature the run starts with
-// or refers to; with the isothermal walls' it sets the unit of temperature,
-// the power of two above every equilibrium g.  Scales far from 1 do not fit
-// the split numbers' exponents: every node then takes the FP64 path (gmax 0).
+// or refers to; with the isothermal walls' it sets the coarsest unit of
+// temperature, the power of two above every equilibrium g.  Scales far from 1 do
+// not fit the split numbers' exponents: every node then takes the FP64 path
+// (gmax 0).  So it does where the largest g at rest, m T with m = max(|sigma -
+// varpi|, varpi / 4), is below T / 32 or sigma T / 32: units that hold T would
+// then hold g to fewer digits than FP64.
 inline SplitPhys split_phys(double sp, double sm, double sv, double s3, double s4, double sigma, double zeta_a,
                             double cT2, double top, const double* uw, const double* vw, const double* Tw,
                             const int* iso) {
@@ -317,29 +365,41 @@ inline SplitPhys split_phys(double sp, double sm, double sv, double s3, double s
     P.c6s = sf_make(2.0 - s3);
     P.cb8 = sf_make(1.0 - 0.5 * s4);
     P.inv_sigma = ratio(1.0, sigma);
-    P.hza = sf_make(0.5 * zeta_a);
     P.kappa = cT2 / sigma;
-    bool fits = true;
+    P.zeta = llrint(ldexp(zeta_a, 61));
+    P.om = (1LL << 61) - P.zeta;
+    const double m = fmax(fabs(sigma - 2.0 * cT2), 0.5 * cT2), tops = sigma > 1.0 ? sigma : 1.0;
+    bool fits = m >= 0.03125 * tops && sigma <= 16.0 && sigma >= 1e-5;
+    frexp(tops / m, &P.ghead);
+    if (!fits || P.ghead < 1) P.ghead = 1;
+    int es = 0;
+    const double is = 1.0 / sigma;
+    frexp(is, &es);                  // is = [1/2, 1) 2^es
+    P.sshift = 3 + es;               // 0 .. 20
+    if (!fits) P.sshift = 0;
+    P.sinv = llrint(ldexp(is, 61 - es)) + llrint(ldexp(::fma(-is, sigma, 1.0) / sigma, 61 - es));
     for (int s = 0; s < 4; ++s) {
         const double t = fabs(Tw[s]);
         fits = fits && t <= 1e300;
         if (iso[s] && t > top) top = t;
     }
-    top *= sigma > 1.0 ? sigma : 1.0;
+    top *= tops;
     fits = fits && top > 1e-18 && top < 1e18;
     int e = 0;
     if (fits) frexp(top, &e);
     P.gexp = e;
-    P.tunit = (float)ldexp(1.0, e);
     P.gmax = fits ? (uint32_t)(1023 + e) << 20 : 0u;
     for (int s = 0; s < 4; ++s) {
-        const double T = fits && iso[s] ? ldexp(Tw[s], -e) : 0.0;
+        const double T = fits && iso[s] ? Tw[s] : 0.0;
+        const bool slow = fabs(uw[s]) < 0.0625 && fabs(vw[s]) < 0.0625;   // else the node is left to the FP64 path
         P.uw[s] = sf_make(uw[s]);
         P.vw[s] = sf_make(vw[s]);
+        P.uwf[s] = slow ? llrint(ldexp(uw[s], 64)) : 0;
+        P.vwf[s] = slow ? llrint(ldexp(vw[s], 64)) : 0;
         P.rest[s] = uw[s] == 0.0 && vw[s] == 0.0;
-        P.Tw[s] = sf_make(T);
-        P.n0w[s] = llrint(ldexp(sigma * T, 60));
-        P.cw[s] = llrint(ldexp(cT2 * T, 60));
+        P.n0w[s] = sigma * T;
+        P.cw[s] = cT2 * T;
+        P.wbig[s] = d_hi(m * fabs(T));
     }
     return P;
 }
@@ -353,13 +413,14 @@ constexpr int kSplitPlanes = 8;
 // Raw moments of Eq. 12 in fixed point, with the O(1) parts removed: three
 // times k20 - rho/3 and so on.  All exact.
 struct FixMom {
-    long long rho, jx, jy, d3, d4, k11, d6, d7, d8, k21, k12;
+    long long rho, jx, jy, d3, d4, k11, d6, d7, d8, k21, k12, k22;
 };
 CLB_SP FixMom fix_moments(const long long (&f)[9]) {
     const long long a = f[5] + f[7], b = f[6] + f[8], c = f[5] - f[7], d = f[6] - f[8];
     const long long s13 = f[1] + f[3], s24 = f[2] + f[4];
     FixMom k;
     const long long k22 = a + b;
+    k.k22 = k22;
     k.k11 = a - b;
     k.k21 = c + d;
     k.k12 = c - d;
@@ -500,49 +561,102 @@ CLB_SP void fix_incr(const Incr8& r, long long (&q)[9], float& worst) {
     to_fix4(pair(r.r5, r.r8), q[5], q[8]);
 }
 
-// Both axes of the temperature collision (see collide5): TU = T u, d = g+ - g-
-// of the pre-collision values.  Returns 2 b, b = (zeta_a / 2)(T u - d), and
-// writes half of s = 2 u h - T u^2 / 2 (h = d / 2 + b; unit shift: T u^2 / 2) in
-// fixed point.
-template <bool SHIFT>
-CLB_SP sf2 split_axes(sf2 TU, sf2 d, sf2 U, const SplitPhys& P, long long (&qs)[2], float& worst) {
-    const sf2 b2 = dbl(mul(both(P.hza), sub(TU, d)));
-    const sf2 hT = scale(TU, 0.5f);
-    const sf2 s2 = dbl(mul(U, SHIFT ? add(d, sub(b2, hT)) : hT));
-    worst = fabs_max(fabs_max(worst, b2.h.x, b2.h.y), s2.h.x, s2.h.y);
-    to_fix4(s2, qs[0], qs[1]);
-    return b2;
+CLB_SP uint32_t hi_word(long long v) { return (uint32_t)((unsigned long long)v >> 32); }
+// What the update of a node is not computed for: k22 of 1 or more (9 k22 could
+// leave 64 bits), a difference D of opposite g of a unit, a density off 1 by an
+// eighth, a temperature of four units, a speed of umax.  (NaN counts as outside.)
+CLB_SP bool split_in_range(const FixMom& k, long long D1, long long D2, sf drho, sf2 U, sf Tn, float umax) {
+    float m = fabs_max(0.0f, U.h.x, U.h.y);
+    m = fabs_max(fmul(m, 1.0f / umax), fmul(drho.h, 8.0f), fmul(Tn.h, 0.25f));
+    return m < 1.0f && hi_word(k.k22) < (1u << 28) && hi_word(D1) + (1u << 28) < (1u << 29) &&
+           hi_word(D2) + (1u << 28) < (1u << 29);
+}
+constexpr float kMaxSpeed = 1.0f / 24;
+
+// 1 + d
+CLB_SP sf one_plus(sf d) {
+    const sf s = quick_sum(1.0f, d.h);
+    return sf{s.h, fadd(s.l, d.l)};
+}
+constexpr long long kOne = 1LL << 60;
+
+// The heat flux T u of a node less its d = g+ - g- (D), both axes, in fixed point.
+// T u / (rho u) = T / rho = T (1 - drho / rho), and rho u = j + p, so the product
+// that is not small is one of two fixed-point numbers, T and j + p; as a split
+// number T u would carry 2^-46 of itself into g, several times what FP64 rounds.
+// n0 = sum g, k.jx, k.jy, D: fixed point; p = rho u - j, also as fixed point (qp:
+// quarters).
+CLB_SP long long split_temperature(long long n0, const SplitPhys& P) {
+    return (long long)((unsigned long long)mul_hi(n0, P.sinv) << P.sshift);
+}
+CLB_SP void split_flux(long long n0, const FixMom& k, long long D1, long long D2, const long long (&qp)[2], sf2 J, sf2 p,
+                       sf Tn, sf drho, sf ir, const SplitPhys& P, long long (&e)[2]) {
+    const long long T = split_temperature(n0, P);
+    long long c1, c2;
+    to_fix4(mul(both(muln(muln(Tn, drho), ir)), add(J, p)), c1, c2);
+    e[0] = mul_hi(T, (long long)((unsigned long long)(k.jx + (qp[0] << 2)) << 4)) - D1 - (c1 << 2);
+    e[1] = mul_hi(T, (long long)((unsigned long long)(k.jy + (qp[1] << 2)) << 4)) - D2 - (c2 << 2);
 }
 
-// One interior node: pre-collision f, g in fixed point in, post-collision out.
-// False: an increment left the range (f and g are then invalid).
+// One interior node: pre-collision f, g in fixed point in, post-collision out;
+// gexp: g's unit (split_unit).  In two parts, so that g can be stored before f is
+// computed (ten registers less through the longer part).  False: not computed (f
+// and g are then invalid).
+struct SplitMid {
+    FixMom k;
+    sf rho;
+    sf2 U, p;
+};
 template <bool SHIFT, bool FORCH>
-CLB_SP bool split_node(long long (&f)[9], long long (&g)[5], const SplitCoef& c, const SplitPhys& P) {
+CLB_SP bool split_heat(const long long (&f)[9], long long (&g)[5], const SplitCoef& c, const SplitPhys& P, int gexp,
+                       float umax, SplitMid& m) {
     const FixMom k = fix_moments(f);
     const long long p1 = g[1] + g[3], p2 = g[2] + g[4], n0 = g[0] + (p1 + p2);
-    const sf2 rn = to_sf2(k.rho, n0);
-    const sf rho = first(rn), ir = recip(rho), Tn = muln(second(rn), P.inv_sigma);
+    const sf2 rn = to_sf2(k.rho - kOne, n0);
+    const sf drho = first(rn), rho = one_plus(drho), ir = recip(rho), Tn = muln(second(rn), P.inv_sigma);
     const sf2 J = to_sf2(k.jx, k.jy);
     sf2 U, hF;
-    split_velocity<FORCH>(ir, J, scale(Tn, P.tunit), c, U, hF);
+    split_velocity<FORCH>(ir, J, scale(Tn, split_tunit(gexp)), c, U, hF);
+    const long long D1 = g[1] - g[3], D2 = g[2] - g[4];
+    if (!split_in_range(k, D1, D2, drho, U, Tn, umax)) return false;
     const sf2 p = mul(both(rho), hF);                     // rho u - j = rho F / 2 by the velocity's definition
-    float worst = 0.0f;
-    // temperature: h3 = c_sT^2 T / 2 + s, and g+ + g- goes to 2 h3 at once
+    float worst = fabs_max(0.0f, p.h.x, p.h.y);
+    long long qp[2];
+    to_fix4(p, qp[0], qp[1]);
+    // temperature (see collide5): g+ - g- goes to d + 2 b, 2 b = zeta_a (T u - d);
+    // h3 = c_sT^2 T / 2 + s, s = 2 u h - T u^2 / 2, h = d / 2 + b (unit shift: T u^2 / 2),
+    // and g+ + g- goes to 2 h3 at once
+    long long e[2], qs[2];
+    split_flux(n0, k, D1, D2, qp, J, p, Tn, drho, ir, P, e);
+    const long long b1 = mul_hi(e[0] << 2, P.zeta), b2 = mul_hi(e[1] << 2, P.zeta);
+    const sf2 hT = scale(mul(both(Tn), U), 0.5f);
+    sf2 s2 = mul(U, SHIFT ? add(hT, to_sf2(b1 + b1 - e[0], b2 + b2 - e[1])) : hT);
+    worst = fabs_max(worst, s2.h.x, s2.h.y);
+    to_fix4(s2, qs[0], qs[1]);
     const long long C = d2ll(ll2d(n0) * P.kappa);
-    long long qs[2], qb[2];
-    to_fix4(split_axes<SHIFT>(muln(both(muln(Tn, ir)), addn(J, p)), to_sf2(g[1] - g[3], g[2] - g[4]), U, P, qs, worst),
-            qb[0], qb[1]);
-    const long long e1 = C - p1 + (qs[0] << 2), e2 = C - p2 + (qs[1] << 2);
-    const long long i1 = (e1 >> 1) + (qb[0] << 1), i2 = (e2 >> 1) + (qb[1] << 1);
+    const long long e1 = C - p1 + (qs[0] << 3), e2 = C - p2 + (qs[1] << 3);
+    const long long i1 = (e1 >> 1) + b1, i2 = (e2 >> 1) + b2;
     g[0] -= e1 + e2;
     g[1] += i1;
     g[3] += e1 - i1;
     g[2] += i2;
     g[4] += e2 - i2;
+    m = SplitMid{k, rho, U, p};
+    return worst < kMaxIncr;
+}
+template <bool SHIFT>
+CLB_SP bool split_flow(long long (&f)[9], const SplitMid& m, sf ip, const SplitPhys& P) {
+    float worst = 0.0f;
     long long q[9];
-    fix_incr(split_collide<SHIFT, true>(split_moments(k, P), rho, U, p, p, c.ip, P), q, worst);
+    fix_incr(split_collide<SHIFT, true>(split_moments(m.k, P), m.rho, m.U, m.p, m.p, ip, P), q, worst);
     fix_apply(f, q);
     return worst < kMaxIncr;
+}
+// Both, in the run's unit and at any speed.
+template <bool SHIFT, bool FORCH>
+CLB_SP bool split_node(long long (&f)[9], long long (&g)[5], const SplitCoef& c, const SplitPhys& P) {
+    SplitMid m;
+    return split_heat<SHIFT, FORCH>(f, g, c, P, P.gexp, 1.0f, m) && split_flow<SHIFT>(f, m, c.ip, P);
 }
 
 // One wall node b by non-equilibrium extrapolation from its inward neighbour
@@ -552,54 +666,72 @@ CLB_SP bool split_node(long long (&f)[9], long long (&g)[5], const SplitCoef& c,
 // n0ss = sum g of the next node inward).
 // REST: the wall does not move (both velocities 0), the usual case; what
 // vanishes then is left out (the wall nodes are a small grid's longest chain).
+// In two parts, as an interior node.
 template <bool SHIFT, bool FORCH, bool REST>
-CLB_SP bool split_wall(long long (&f)[9], long long (&g)[5], long long n0ss, const SplitCoef& cs, const SplitCoef& cb,
-                       int side_u, int side_t, const SplitPhys& P) {
+CLB_SP bool split_wall_heat(const long long (&f)[9], long long (&g)[5], long long n0ss, const SplitCoef& cs, int side_u,
+                            int side_t, const SplitPhys& P, int gexp, float umax, SplitMid& m, sf& Tb) {
     const FixMom k = fix_moments(f);
     const long long n0s = g[0] + ((g[1] + g[3]) + (g[2] + g[4]));
-    const sf2 rn = to_sf2(k.rho, n0s);
-    const sf rho = first(rn), Tsn = muln(second(rn), P.inv_sigma);
+    const sf2 rn = to_sf2(k.rho - kOne, n0s);
+    const sf drho = first(rn), rho = one_plus(drho), ir = recip(rho), Tsn = muln(second(rn), P.inv_sigma);
+    const sf2 J = to_sf2(k.jx, k.jy);
     sf2 U, hF;
-    split_velocity<FORCH>(recip(rho), to_sf2(k.jx, k.jy), scale(Tsn, P.tunit), cs, U, hF);
+    split_velocity<FORCH>(ir, J, scale(Tsn, split_tunit(gexp)), cs, U, hF);
+    const long long D1 = g[1] - g[3], D2 = g[2] - g[4];
+    if (!split_in_range(k, D1, D2, drho, U, Tsn, umax)) return false;
     const sf2 p = mul(both(rho), hF);                     // rho u - j, the same at s and b
     const sf2 uw = pair(P.uw[side_u], P.vw[side_u]);
+    float worst = fabs_max(0.0f, p.h.x, p.h.y);
+    if constexpr (!REST) {
+        if (!(fabs_max(0.0f, uw.h.x, uw.h.y) < fmin_f(umax, 0.0625f))) return false;
+    }
     long long n0, C;
-    sf Tn;
     if (side_t >= 0) {
-        n0 = P.n0w[side_t];
-        C = P.cw[side_t];
-        Tn = P.Tw[side_t];
+        n0 = fix_d(P.n0w[side_t], gexp);
+        C = fix_d(P.cw[side_t], gexp);
     } else {
         n0 = n0s + d2ll(ll2d(n0s - n0ss) * (1.0 / 3.0));
         C = d2ll(ll2d(n0) * P.kappa);
-        Tn = muln(first(to_sf2(n0, n0)), P.inv_sigma);
     }
-    float worst = 0.0f;
-    // temperature: d = g+ - g- at b is its value at s plus T_b u_w - T_s u_s
-    const long long D1 = g[1] - g[3], D2 = g[2] - g[4];
-    long long qs[2] = {0, 0}, qv[2];
-    sf2 v;
-    if constexpr (REST) {   // T_b u_w = 0: s = 0, 2 b = -zeta_a d
-        const sf2 t = neg(mul(both(Tsn), U));
-        v = dbl(fnma(both(dbl(P.hza)), add(to_sf2(D1, D2), t), t));
-    } else {
-        const sf2 TU = mul(both(Tn), uw), t = fnma(both(Tsn), U, TU);
-        v = dbl(add(split_axes<SHIFT>(TU, add(to_sf2(D1, D2), t), uw, P, qs, worst), t));
+    const sf Tn = muln(first(to_sf2(n0, n0)), P.inv_sigma);
+    worst = fabs_max(worst, fmul(Tn.h, 0.25f * kMaxIncr), 0.0f);
+    // temperature: d = g+ - g- at b is its value at s plus T_b u_w - T_s u_s, and
+    // goes to T_b u_w + (1 - zeta_a) (d_s - T_s u_s)
+    long long qp[2], e[2], qs[2] = {0, 0}, W1 = 0, W2 = 0;
+    to_fix4(p, qp[0], qp[1]);
+    split_flux(n0s, k, D1, D2, qp, J, p, Tsn, drho, ir, P, e);
+    const long long v1 = mul_hi(e[0] << 2, P.om) << 1, v2 = mul_hi(e[1] << 2, P.om) << 1;   // (1 - zeta_a) e
+    if constexpr (!REST) {
+        const long long T = split_temperature(n0, P);
+        W1 = mul_hi(T, P.uwf[side_u]);
+        W2 = mul_hi(T, P.vwf[side_u]);
+        const sf2 hT = scale(mul(both(Tn), uw), 0.5f), s2 = mul(uw, SHIFT ? sub(hT, to_sf2(v1, v2)) : hT);
+        worst = fabs_max(worst, s2.h.x, s2.h.y);
+        to_fix4(s2, qs[0], qs[1]);
     }
-    worst = fabs_max(worst, v.h.x, v.h.y);
-    to_fix4(v, qv[0], qv[1]);
-    const long long e1 = C + (qs[0] << 2), e2 = C + (qs[1] << 2);
+    const long long e1 = C + (qs[0] << 3), e2 = C + (qs[1] << 3);
     g[0] = n0 - e1 - e2;
-    g[1] = (e1 + D1 + (qv[0] << 1)) >> 1;
+    g[1] = (e1 + W1 - v1) >> 1;
     g[3] = e1 - g[1];
-    g[2] = (e2 + D2 + (qv[1] << 1)) >> 1;
+    g[2] = (e2 + W2 - v2) >> 1;
     g[4] = e2 - g[2];
-    // flow: moments of b minus those of s, and the collision's increments at b
+    m = SplitMid{k, rho, U, p};
+    Tb = scale(Tn, split_tunit(gexp));
+    return worst < kMaxIncr;
+}
+template <bool SHIFT, bool FORCH, bool REST>
+CLB_SP bool split_wall_flow(long long (&f)[9], const SplitMid& s, sf Tb, sf ips, const SplitCoef& cb, int side_u,
+                            const SplitPhys& P) {
+    const FixMom& k = s.k;
+    const sf rho = s.rho;
+    const sf2 U = s.U, p = s.p, uw = pair(P.uw[side_u], P.vw[side_u]);
+    float worst = 0.0f;
+    // moments of b minus those of s, and the collision's increments at b
     SplitMom m = split_moments(k, P);
     sf2 m34, ru;
     sf m5, m8;
     Incr8 r;
-    const sf2 RU = mul(both(rho), U), IU = mul(both(cs.ip), U);
+    const sf2 RU = mul(both(rho), U), IU = mul(both(ips), U);
     const sf sXY = mul(first(IU), second(RU)), sq = mul(sXY, mul(first(IU), second(U)));
     if constexpr (REST) {
         m34 = neg(mul(IU, RU));
@@ -609,7 +741,7 @@ CLB_SP bool split_wall(long long (&f)[9], long long (&g)[5], long long n0ss, con
         m.a67 = fnma(both(sXY), U, m.a67);
         m.a5 = add(m.a5, m5);
         m.a8 = add(m.a8, m8);
-        const sf2 F = mul(both(rho), pair(cb.hgx, fma(cb.hgb, scale(Tn, P.tunit), cb.hgy)));
+        const sf2 F = mul(both(rho), pair(cb.hgx, fma(cb.hgb, Tb, cb.hgy)));
         r.r12 = add(p, F);
         r.r34 = neg(fma(both(P.sp), m.a34, mul(both(P.sm), swp(m.a34))));
         r.r5 = neg(mul(P.sv, m.a5));
@@ -627,14 +759,14 @@ CLB_SP bool split_wall(long long (&f)[9], long long (&g)[5], long long n0ss, con
         m.a67 = add(m.a67, sub(mul(both(wXY), uw), mul(both(sXY), U)));
         m.a5 = add(m.a5, m5);
         m.a8 = add(m.a8, m8);
-        const sf2 Fb = mul(both(rho), split_force<FORCH>(uw, scale(Tn, P.tunit), cb));
+        const sf2 Fb = mul(both(rho), split_force<FORCH>(uw, Tb, cb));
         r = split_collide<SHIFT, false>(m, rho, uw, p, Fb, cb.ip, P);
     }
     // increments against s: the first-order rows and j / 3 of rows 6, 7 are
-    // replaced outright (their values at s go out in fixed point)
+    // replaced outright (their values at s go out, and rho u_w comes in, in fixed point)
     sf2 j = neg(p);
-    if constexpr (!REST) j = sub(ru, p);
     r.r12 = add(r.r12, j);
+    if constexpr (!REST) j = add(j, ru);
     r.r34 = add(r.r34, m34);
     r.r5 = add(r.r5, m5);
     r.r67 = add(r.r67, fma(both(P.third), swp(j), m.a67));
@@ -643,10 +775,14 @@ CLB_SP bool split_wall(long long (&f)[9], long long (&g)[5], long long n0ss, con
     fix_incr(r, q, worst);
     q[1] -= (k.jx + 2) >> 2;
     q[2] -= (k.jy + 2) >> 2;
+    if constexpr (!REST) {
+        q[1] += mul_hi(k.rho, P.uwf[side_u]) >> 2;
+        q[2] += mul_hi(k.rho, P.vwf[side_u]) >> 2;
+    }
     q[6] -= (k.k21 + 2) >> 2;
     q[7] -= (k.k12 + 2) >> 2;
     fix_apply(f, q);
-    return worst < kMaxIncr;
+    return worst < (REST ? kMaxIncr : 2.0f * kMaxIncr);   // j / 3 alone takes half of that
 }
 
 }  // namespace clb
