@@ -60,8 +60,9 @@ struct clb_handle {
     uint2* rec[2] = {nullptr, nullptr};   // FP16N form: per-node baseline record
     unsigned* seq = nullptr;              // FP16 forms: step counter of each buffer (seeds the rounding)
     int par = 0;
-    CoefT<double>* coef = nullptr;   // FP64 form: per-node constants
+    Coef4* coef = nullptr;           // FP64 form: per-node constants
     float2* scoef = nullptr;         // and as split numbers, in planes
+    float2* sayg = nullptr;          // ayg as split numbers
     float* phi32 = nullptr;          // FP16 forms: porosity (dense) or 1/phi (pitched)
     void* ayg = nullptr;             // a_y - g beta T0 per row (double or float)
     double* scratch = nullptr;       // 4 dense fields (macros, set_fields)
@@ -84,7 +85,7 @@ struct clb_handle {
     unsigned* tma_fail = nullptr;   // device flag set by a CTA whose wait expired
     std::string err;
 
-    AuxT<double> aux64() const { return AuxT<double>{coef, nullptr, nullptr, (const double*)ayg, scoef}; }
+    AuxT<double> aux64() const { return AuxT<double>{coef, nullptr, nullptr, (const double*)ayg, scoef, sayg}; }
     AuxT<float> aux32() const {
         return prec == CLB_F16N ? AuxT<float>{nullptr, nullptr, phi32, (const float*)ayg}
                                 : AuxT<float>{nullptr, phi32, nullptr, (const float*)ayg};
@@ -333,6 +334,7 @@ static void free_all(clb_handle* h) {
     cudaFree(h->seq);
     cudaFree(h->coef);
     cudaFree(h->scoef);
+    cudaFree(h->sayg);
     cudaFree(h->phi32);
     cudaFree(h->ayg);
     cudaFree(h->scratch);
@@ -629,6 +631,8 @@ extern "C" int clb_init(clb_handle** out, const clb_params* p, const double* phi
     h->sp = split_phys(h->k64.p.sp, h->k64.p.sm, lat.sv, p->s3, p->s4, p->sigma, lat.zeta_a, h->k64.p.cT2,
                        std::max(std::fabs(p->T0) + p->dT, std::fabs(p->T_init)), h->k64.b.uw, h->k64.b.vw, h->k64.b.Tw,
                        h->k64.b.iso);
+    h->sp.ax = sf_make(p->ax);
+    h->sp.gbeta = sf_make(lat.gbeta);
     pick_launch(h);
 
     const size_t fbytes = (size_t)G.plane * 9 * h->es;
@@ -655,7 +659,8 @@ extern "C" int clb_init(clb_handle** out, const clb_params* p, const double* phi
         CKI(cudaMalloc(&h->phi32, (size_t)G.plane * sizeof(float)));
         CKI(cudaMemsetAsync(h->phi32, 0, (size_t)G.plane * sizeof(float), h->stream));
     } else {
-        CKI(cudaMalloc(&h->coef, (size_t)n * sizeof(CoefT<double>)));
+        CKI(cudaMalloc(&h->coef, (size_t)n * sizeof(Coef4)));
+        CKI(cudaMalloc(&h->sayg, (size_t)p->ny * sizeof(float2)));
         CKI(cudaMalloc(&h->scoef, (size_t)n * sizeof(float2) * kSplitPlanes));
     }
     CKI(cudaMalloc(&h->ayg, (size_t)p->ny * (half ? sizeof(float) : sizeof(double))));
@@ -681,10 +686,9 @@ extern "C" int clb_init(clb_handle** out, const clb_params* p, const double* phi
         k_phi32<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->scratch, h->phi32, p->nx, p->ny, px,
                                                                       h->prec == CLB_F16N);
     else {
-        k_coef<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->scratch, (const double*)h->ayg, h->coef,
-                                                                     p->nx, n, lat.nu, lat.K, p->ax, lat.gbeta,
-                                                                     p->forchheimer);
-        k_split_coef<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->coef, h->scoef, n);
+        k_coef<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->scratch, h->coef, n, lat.nu, lat.K, p->forchheimer);
+        k_split_coef<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(h->coef, h->scoef, n,
+                                                                           (const double*)h->ayg, h->sayg, p->ny);
     }
     CKI(cudaGetLastError());
     CKI(cudaStreamSynchronize(h->stream));

@@ -73,6 +73,12 @@ struct alignas(8 * sizeof(R)) CoefT {
     R hgy;   // phi (a_y - g beta T0) / 2 of the node's row
 };
 
+// The four of them the FP64 form keeps per node; the others are products with the
+// run's or the row's constants (coef_from4).
+struct alignas(32) Coef4 {
+    double ip, hdar, aux, hp;   // hp = phi / 2
+};
+
 struct Geo {
     int nx, ny, px;       // grid and row pitch (elements)
     long long plane;      // px * ny
@@ -121,11 +127,12 @@ struct AuxT {
 };
 template <>
 struct AuxT<double> {
-    const CoefT<double>* coef;
+    const Coef4* coef;
     const float* phi;
     const float* ip;
     const double* ayg;
     const float2* scoef;   // the constants as split numbers, kSplitPlanes dense planes
+    const float2* sayg;    // ayg as split numbers
 };
 
 // One ping-pong buffer: distribution planes, and for the equilibrium-shifted
@@ -731,6 +738,13 @@ __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// All constants of a node (the products rounded on their own, not fused into a sum).
+__device__ __forceinline__ CoefT<double> coef_from4(const Coef4& c, double ayg, const PhysT<double>& P) {
+    const double l0 = 0.5 + 0.5 * c.hdar;                             // Eq. 23
+    return CoefT<double>{c.ip, l0, __dmul_rn(l0, l0), c.aux, c.hdar, __dmul_rn(c.hp, P.ax), __dmul_rn(c.hp, P.gbeta),
+                         __dmul_rn(c.hp, ayg)};
+}
+
 // A storage policy reads the streamed values of a node (pull9 / pull5),
 // writes a node's post-collision values (store) and gives the per-node
 // constants (coef).  L: how the distribution buffers are loaded.
@@ -782,7 +796,7 @@ struct StoreF64T {
     }
     template <bool FORCH>
     static __device__ __forceinline__ CoefT<R> coef(const AuxT<R>& A, const KParamsT<R>& K, int x, int y) {
-        return A.coef[(long long)y * K.g.nx + x];
+        return coef_from4(A.coef[(long long)y * K.g.nx + x], A.ayg[y], K.p);
     }
 };
 
@@ -1377,7 +1391,7 @@ __device__ __forceinline__ void wall_node(const Geo& G, int i, int& x, int& y) {
 // buffers and loads as step_interior / step_wall, the arithmetic on the FP32
 // and integer pipes.  False: the node left the fixed-point range and has not
 // been stored; the caller takes the FP64 path for it.
-__device__ __forceinline__ SplitCoef split_coef(const AuxT<double>& A, const Geo& G, int x, int y) {
+__device__ __forceinline__ SplitCoef split_coef(const AuxT<double>& A, const Geo& G, const SplitPhys& P, int x, int y) {
     const long long n = (long long)G.nx * G.ny;
     const float2* p = A.scoef + ((long long)y * G.nx + x);
     sf v[kSplitPlanes];
@@ -1386,7 +1400,8 @@ __device__ __forceinline__ SplitCoef split_coef(const AuxT<double>& A, const Geo
         const float2 t = __ldg(p + k * n);
         v[k] = sf{t.x, t.y};
     }
-    return SplitCoef{v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]};
+    const float2 ay = __ldg(A.sayg + y);
+    return split_coef_from4(v[0], v[1], v[2], v[3], sf{ay.x, ay.y}, P);
 }
 
 // The values a node is computed from: f in fixed point (range: see fix_f), g as
@@ -1426,7 +1441,7 @@ __device__ __forceinline__ bool split_step_interior(const BufT<double>& in, cons
     long long f[9], g[5];
     double vg[5];
     uint32_t range = 0u, big = 0u;
-    const SplitCoef c = split_coef(A, G, x, y);
+    const SplitCoef c = split_coef(A, G, P, x, y);
     split_pull<L>(in, G, x, y, f, vg, range, big);
     const int gexp = split_unit(big, P);
 #pragma unroll
@@ -1460,7 +1475,7 @@ __device__ __forceinline__ bool split_step_wall(const BufT<double>& in, const Bu
     double vg[5], vs[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     uint32_t range = 0u, big = w.st < 0 ? 0u : P.wbig[w.st];
     const int sx = x + w.dx, sy = y + w.dy;
-    const SplitCoef cs = split_coef(A, G, sx, sy), cb = split_coef(A, G, x, y);
+    const SplitCoef cs = split_coef(A, G, P, sx, sy), cb = split_coef(A, G, P, x, y);
     split_pull<L>(in, G, sx, sy, f, vg, range, big);
     if (w.st < 0) {
         long long o[9];
@@ -2046,38 +2061,39 @@ __global__ void k_fill4(double* __restrict__ d, long long n, double a, double b,
 
 // Per-node FP64 constants from the porosity (Eqs. 4, 5, 23) and the row's
 // a_y - g beta T0 (ayg, one value per row).
-__global__ void k_coef(const double* __restrict__ phi, const double* __restrict__ ayg, CoefT<double>* __restrict__ coef,
-                       int nx, long long n, double nu, double K, double ax, double gbeta, int forch) {
+__global__ void k_coef(const double* __restrict__ phi, Coef4* __restrict__ coef, long long n, double nu, double K, int forch) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double p = phi[i], hp = 0.5 * p;
-    CoefT<double> c;
+    const double p = phi[i];
+    Coef4 c;
+    c.hp = 0.5 * p;
     c.ip = 1.0 / p;
-    c.hdar = hp * nu / K;
-    c.l0 = 0.5 + 0.5 * c.hdar;                                   // Eq. 23
-    c.l0sq = c.l0 * c.l0;
+    c.hdar = c.hp * nu / K;
     if (forch) {
         const double Fphi = 1.75 / sqrt(150.0 * p * p * p);      // Ergun, Eq. 5
         c.aux = 0.5 * p * Fphi / sqrt(K);                         // l1 of Eq. 23
     } else {
-        c.aux = 1.0 / (2.0 * c.l0);                               // 1 / (2 l0), Eq. 23
+        c.aux = 1.0 / (2.0 * (0.5 + 0.5 * c.hdar));               // 1 / (2 l0), Eq. 23
     }
-    c.hgx = hp * ax;
-    c.hgb = hp * gbeta;
-    c.hgy = hp * ayg[i / nx];
     coef[i] = c;
 }
 
-// The same constants as split numbers, in planes (see SplitCoef).
-__global__ void k_split_coef(const CoefT<double>* __restrict__ coef, float2* __restrict__ out, long long n) {
+// The same constants as split numbers, in planes (see split_coef_from4), and
+// the rows' a_y - g beta T0.
+__global__ void k_split_coef(const Coef4* __restrict__ coef, float2* __restrict__ out, long long n,
+                             const double* __restrict__ ayg, float2* __restrict__ sayg, int ny) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const CoefT<double> c = coef[i];
-    const double v[kSplitPlanes] = {c.ip, c.l0, c.l0sq, c.aux, c.hdar, c.hgx, c.hgb, c.hgy};
+    const Coef4 c = coef[i];
+    const double v[kSplitPlanes] = {c.ip, c.hdar, c.aux, c.hp};
 #pragma unroll
     for (int k = 0; k < kSplitPlanes; ++k) {
         const sf s = sf_make(v[k]);
         out[k * n + i] = make_float2(s.h, s.l);
+    }
+    if (i < ny) {
+        const sf s = sf_make(ayg[i]);
+        sayg[i] = make_float2(s.h, s.l);
     }
 }
 

@@ -301,6 +301,7 @@ struct SplitPhys {
     sf ca2, c6s, cb8;                // unit shift: 2 (1 - s_v/2), 2 (1 - s3/2), 1 - s4/2
     sf inv_sigma;                    // 1 / sigma
     double kappa;                    // c_sT^2 / sigma
+    sf ax, gbeta;                    // body force, g beta (set by the run, see split_coef_from4)
     long long sinv;                  // 2^(64 - sshift) / sigma, in [2^60, 2^61]
     int sshift;
     long long zeta, om;              // zeta_a, 1 - zeta_a in units of 2^-61
@@ -408,7 +409,14 @@ inline SplitPhys split_phys(double sp, double sm, double sv, double s3, double s
 struct SplitCoef {
     sf ip, l0, l0sq, aux, hdar, hgx, hgb, hgy;
 };
-constexpr int kSplitPlanes = 8;
+// From the four a run keeps (1/phi, phi nu / (2 K), aux, phi / 2; 32 bytes a node,
+// as many as their FP64 forms), the row's a_y - g beta T0 and the run's a_x, g beta.
+constexpr int kSplitPlanes = 4;
+CLB_SP SplitCoef split_coef_from4(sf ip, sf hdar, sf aux, sf hp, sf ayg, const SplitPhys& P) {
+    const sf h = scale(hdar, 0.5f), s = two_sum(0.5f, h.h), l0 = norm(sf{s.h, fadd(s.l, h.l)});
+    const sf2 hg = mul(both(hp), pair(P.ax, ayg));
+    return SplitCoef{ip, l0, mul(l0, l0), aux, hdar, first(hg), mul(hp, P.gbeta), second(hg)};
+}
 
 // Raw moments of Eq. 12 in fixed point, with the O(1) parts removed: three
 // times k20 - rho/3 and so on.  All exact.
