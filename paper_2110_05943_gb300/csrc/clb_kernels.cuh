@@ -1443,11 +1443,12 @@ __device__ __forceinline__ bool split_step_interior(const BufT<double>& in, cons
     uint32_t range = 0u, big = 0u;
     const SplitCoef c = split_coef(A, G, P, x, y);
     split_pull<L>(in, G, x, y, f, vg, range, big);
+    if (!(fix_ok(range) && big < P.gmax)) return false;
     const int gexp = split_unit(big, P);
 #pragma unroll
     for (int i = 0; i < 5; ++i) g[i] = fix_d(vg[i], gexp);
     SplitMid m;
-    if (!(split_heat<SHIFT, FORCH>(f, g, c, P, gexp, kMaxSpeed, m) && fix_ok(range) && big < P.gmax)) return false;
+    if (!split_heat<SHIFT, FORCH>(f, g, c, P, gexp, kMaxSpeed, m)) return false;
     split_store_g(out, G, gexp, x, y, g);
     if (!split_flow<SHIFT>(f, m, c.ip, P)) return false;
     split_store_f(out, G, x, y, f);
