@@ -206,8 +206,8 @@ static int map_params(const clb_params* p, clb_lattice* lat, std::string& why) {
     return CLB_OK;
 }
 
-// Block shapes: 64 x 2 threads for both, one node per thread (FP64) or a
-// node pair (FP16: 128 x 2 nodes, each warp a 128-byte line of every FP16
+// Block shapes: 64 x 1 threads, one node per thread (FP64), or 64 x 2, a
+// node pair per thread (FP16: 128 x 2 nodes, each warp a 128-byte line of every FP16
 // plane).  Measured at 8192^2 with 7 rest-shifted blocks per SM: F16S
 // 78.0 GLUPS with 64-wide blocks, 77.4 with 32 x 4, 76.0 with 16 x 8, 54.6
 // with 8 x 16, 78.1 with 128 x 1; F16N 46.7, 46.7, 46.6, 42.5, 46.6.  On
@@ -455,8 +455,8 @@ static void macros_as(clb_handle* h, const AuxT<typename P::R>& A, const K& kp, 
                       double* T, unsigned long long* bad) {
     using S = typename P::S;
     const BufT<S> in = h->buf<S>(h->par);
-    if (h->prm.forchheimer) k_macros<P, true><<<h->grid, h->block, 0, h->stream>>>(in, A, kp, r, u, v, T, bad);
-    else k_macros<P, false><<<h->grid, h->block, 0, h->stream>>>(in, A, kp, r, u, v, T, bad);
+    if (h->prm.forchheimer) k_macros<P, true><<<h->grid.x * h->grid.y, h->block, 0, h->stream>>>(in, A, kp, r, u, v, T, bad);
+    else k_macros<P, false><<<h->grid.x * h->grid.y, h->block, 0, h->stream>>>(in, A, kp, r, u, v, T, bad);
 }
 
 static void launch_macros(clb_handle* h, double* r, double* u, double* v, double* T,
@@ -469,7 +469,7 @@ static void launch_macros(clb_handle* h, double* r, double* u, double* v, double
 template <class P, typename K>
 static void set_fields_as(clb_handle* h, const AuxT<typename P::R>& A, const K& kp, const double* d, long long n) {
     using S = typename P::S;
-    k_set_fields<P><<<h->grid, h->block, 0, h->stream>>>(h->buf<S>(0), A, d, d + n, d + 2 * n, d + 3 * n, kp);
+    k_set_fields<P><<<h->grid.x * h->grid.y, h->block, 0, h->stream>>>(h->buf<S>(0), A, d, d + n, d + 2 * n, d + 3 * n, kp);
 }
 
 template <class P, typename K>

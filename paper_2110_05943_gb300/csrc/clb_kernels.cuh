@@ -1982,6 +1982,15 @@ __global__ void __launch_bounds__(128, CLB_BATCH_MINB)
     }
 }
 
+// The thread's node where a one-dimensional grid of blocks covers all nodes in rows
+// of tiles (two grid dimensions would hold ny below 65536 rows of blocks).
+__device__ __forceinline__ bool block_node(const Geo& G, int& x, int& y) {
+    const unsigned tx = (unsigned)(G.nx + blockDim.x - 1) / blockDim.x;
+    x = (int)(blockIdx.x % tx * blockDim.x + threadIdx.x);
+    y = (int)(blockIdx.x / tx * blockDim.y + threadIdx.y);
+    return x < G.nx && y < G.ny;
+}
+
 // Macroscopic fields at the current time level (dense ny*nx FP64 outputs),
 // and (bad not NULL) the first node whose fields are not all finite.
 template <class P, bool FORCH>
@@ -1989,9 +1998,8 @@ __global__ void k_macros(const BufT<typename P::S> in, const AuxT<typename P::R>
                          const KParamsT<typename P::R> K, double* __restrict__ orho, double* __restrict__ oux,
                          double* __restrict__ ouy, double* __restrict__ oT, unsigned long long* __restrict__ bad) {
     using R = typename P::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= K.g.nx || y >= K.g.ny) return;
+    int x, y;
+    if (!block_node(K.g, x, y)) return;
     const long long n = (long long)y * K.g.nx + x;
     const CoefT<R> c = P::template coef<FORCH>(A, K, x, y);
     R f[9], g[5], rho, X, Y, T, Tt, hFx, hFy, n0;
@@ -2017,9 +2025,8 @@ __global__ void k_set_fields(const BufT<typename P::S> out, const AuxT<typename 
                              const double* __restrict__ uy, const double* __restrict__ T,
                              const KParamsT<typename P::R> K) {
     using R = typename P::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= K.g.nx || y >= K.g.ny) return;
+    int x, y;
+    if (!block_node(K.g, x, y)) return;
     const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
     const int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
     R f[9], g[5];
