@@ -1457,6 +1457,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tma(const __grid_constant_
 //   dy  the N columns are those of up to three dY rows, neighbours in the ring
 //       (dY rows y - 1, y, y + 1 meet X row y at the taps dy = 1, 0, -1); two
 //       MMAs where the ring wraps between them or three rows exceed N = 256.
+//       Rows outside the image are left out, not taken as zeros: an infinite X in
+//       the first or last row must not reach the taps that do not contain it.
+//       So the accumulators start from zeros stored to TMEM.
 // The thread that issues the MMAs bounds this kernel (it took the same time
 // without its copies, and half without its MMAs), hence few wide MMAs and a loop
 // over constant offsets (wr_row).  A first form kept three X rows and took an MMA
@@ -1476,21 +1479,28 @@ __device__ __forceinline__ void red_add4(float* p, float a, float b, float c, fl
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
+// 32 columns of this warp's 32 TMEM lanes set to zero (no wait).
+__device__ __forceinline__ void tc_st32_zero(uint32_t taddr) {
+    const uint32_t z = 0u;
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1,"
+        " %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr), "r"(z)
+        : "memory");
+}
+
 // The MMAs of one X row: `ksteps` steps of 16 pixels, NC atoms, in one or two
-// column groups (the second starts at column d2).
+// column groups (the second starts d2 columns after the first, which starts at tmem).
 template <int NC, bool TWO>
 __device__ __forceinline__ void wr_row(uint32_t tmem, uint32_t al, uint32_t b1, uint32_t b2, uint32_t bhi, uint32_t id1,
-                                       uint32_t id2, int tile_n, uint32_t d2, uint32_t xj, int bstep, int ksteps,
-                                       uint32_t acc) {
+                                       uint32_t id2, int tile_n, uint32_t d2, uint32_t xj, int bstep, int ksteps) {
 #pragma unroll 2
     for (int ks = 0; ks < ksteps; ++ks) {
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
             const uint32_t d = tmem + (uint32_t)(3 * tile_n * j), a = al + (uint32_t)(64 * ks) + xj * j;
-            tc_mma_lo(d, a, desc_hi(64), b1 + (uint32_t)(bstep * ks), bhi, id1, acc);
-            if (TWO) tc_mma_lo(d + d2, a, desc_hi(64), b2 + (uint32_t)(bstep * ks), bhi, id2, acc);
+            tc_mma_lo(d, a, desc_hi(64), b1 + (uint32_t)(bstep * ks), bhi, id1, 1u);
+            if (TWO) tc_mma_lo(d + d2, a, desc_hi(64), b2 + (uint32_t)(bstep * ks), bhi, id2, 1u);
         }
-        acc = 1;
     }
 }
 
@@ -1545,8 +1555,13 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     pdl_start();   // every CTA holds its TMEM (see k_conv_tma)
-    pdl_wait();
     const uint32_t tmem = *tmem_slot;
+    for (int c0 = 0; c0 < tmem_cols; c0 += 32) tc_st32_zero(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    pdl_wait();
 
     // Both issuers walk the same items: for every run of rows [ya, yb) within
     // an image, dY rows ya - 1 .. yb, and with dY row y + 1 the X row y.
@@ -1584,7 +1599,6 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
         const uint32_t d_bias = tmem + (uint32_t)(3 * na * tile_n);
         const int maxr = min(3, 256 / tile_n);
         int it = 0, st = 0, ph = 0;
-        uint32_t acc = 0;
         for (int r = r0; r < r1 && ok;) {
             const int img = r / s.h, ya = r - img * s.h, yb = min(s.h, ya + (r1 - r));
             int p1 = 0, p2 = 0;   // the stages one and two items back
@@ -1595,30 +1609,30 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_row(const __grid_constant_
                 }
                 if (x > ya) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    // the first k1 of the three dY rows lie one after the other from p2 on
-                    const int k1 = min(maxr, st >= 2 ? 3 : 2 - st), q = p2 + k1 >= stages ? p2 + k1 - stages : p2 + k1;
-                    const uint32_t id1 = tc_idesc(k1 * tile_n) | mn, id2 = tc_idesc((3 - k1) * tile_n) | mn;
-                    const uint32_t al = x_lo + (uint32_t)(st * (xs >> 4));
-                    const uint32_t b1 = y_lo + (uint32_t)(p2 * (ys >> 4)), b2 = y_lo + (uint32_t)(q * (ys >> 4));
+                    // dY rows y - 1 .. y + 1 within the image: column groups lo .. lo + nr - 1, in the
+                    // ring from stage s0 on; the first k1 of them lie one after the other
+                    const int y = x - 1, lo = y == 0, nr = (y == s.h - 1 ? 2 : 3) - lo;
+                    const int s0 = p2 + lo >= stages ? p2 + lo - stages : p2 + lo;
+                    const int k1 = min(min(maxr, nr), stages - s0), q = s0 + k1 >= stages ? s0 + k1 - stages : s0 + k1;
+                    const uint32_t id1 = tc_idesc(k1 * tile_n) | mn, id2 = tc_idesc(max(1, nr - k1) * tile_n) | mn;
+                    const uint32_t al = x_lo + (uint32_t)(st * (xs >> 4)), d1 = tmem + (uint32_t)(lo * tile_n);
+                    const uint32_t b1 = y_lo + (uint32_t)(s0 * (ys >> 4)), b2 = y_lo + (uint32_t)(q * (ys >> 4));
                     const uint32_t d2 = (uint32_t)(k1 * tile_n), xj = (uint32_t)(x_bytes >> 4);
-                    if (k1 == 3) {
-                        if (nc == 1) wr_row<1, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
-                        else if (nc == 2) wr_row<2, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
-                        else if (nc == 3) wr_row<3, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
-                        else wr_row<4, false>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                    if (k1 == nr) {
+                        if (nc == 1) wr_row<1, false>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
+                        else if (nc == 2) wr_row<2, false>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
+                        else if (nc == 3) wr_row<3, false>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
+                        else wr_row<4, false>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
                     } else {
-                        if (nc == 1) wr_row<1, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
-                        else if (nc == 2) wr_row<2, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
-                        else if (nc == 3) wr_row<3, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
-                        else wr_row<4, true>(tmem, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps, acc);
+                        if (nc == 1) wr_row<1, true>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
+                        else if (nc == 2) wr_row<2, true>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
+                        else if (nc == 3) wr_row<3, true>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
+                        else wr_row<4, true>(d1, al, b1, b2, bhi, id1, id2, tile_n, d2, xj, 2 * bw, ksteps);
                     }
                     if (bias)
-                        for (int ks = 0; ks < ksteps; ks += bm) {
+                        for (int ks = 0; ks < ksteps; ks += bm)
                             tc_mma_lo(d_bias, ones_lo, desc_hi(64), bias_lo + (uint32_t)(p1 * (ys >> 4) + ks * 2 * bw), bhi,
-                                      tc_idesc(min(bm, ksteps - ks) * tile_n) | mn, acc);
-                            acc = 1;
-                        }
-                    acc = 1;
+                                      tc_idesc(min(bm, ksteps - ks) * tile_n) | mn, 1u);
                     tc_commit(smem_u32(&empty[p2]));
                     if (x == yb) {   // the run's last rows are free too
                         tc_commit(smem_u32(&empty[p1]));
