@@ -54,3 +54,18 @@ def test_infinities_at_the_border(lib, n, h, w, ci, co, row, splitk):
     err = (dw.double() - want)[~reached].abs().max()
     assert float(err) <= 1e-5 * float(want.abs().max())
     assert float((db.double() - dy.double().sum((0, 1, 2))).abs().max()) <= 1e-5 * float(dy.double().sum((0, 1, 2)).abs().max())
+
+
+@pytest.mark.parametrize("ci,co", [(160, 160), (288, 160), (192, 192), (288, 96)])
+def test_wide_layers_with_many_pixels(lib, ci, co):
+    """16 x 128^2 pixels, the library's split.  An accumulator of m products of unit
+    variance in FP32 is off by at most 2^-24 sqrt(m) per addition in its size and adds m / 16
+    times: at m = 20,000 that stays below 1e-5 of the largest sum over 262,144 pixels (about
+    5 x 512) -- the bound the narrow layers are held to."""
+    g = torch.Generator(device="cuda").manual_seed(6)
+    x = torch.randn((16, 128, 128, ci), generator=g, device="cuda").bfloat16()
+    dy = torch.randn((16, 128, 128, co), generator=g, device="cuda").bfloat16()
+    dw, db = _run(lib, x, dy, 0)
+    want = _wgrad64(x, dy)
+    assert float((dw.double() - want).abs().max()) <= 1e-5 * float(want.abs().max())
+    assert float((db.double() - dy.double().sum((0, 1, 2))).abs().max()) <= 1e-5 * float(dy.double().sum((0, 1, 2)).abs().max())
