@@ -2021,10 +2021,10 @@ bool launch_wgrad_row(const void* x, const void* dy, float* dw, float* db, ConvS
     const int least = std::max(4, na * tile_n / 12);
     long long gz = splitk >= 1 ? splitk : std::max(1, sm_count() / (groups * ntn));
     gz = std::max(1LL, std::min(gz, splitk >= 1 ? (long long)rows : (long long)(rows + least - 1) / least));
-    // and at most 8192 pixels in an accumulator: wide layers have many tiles and so few
-    // splits, and an FP32 sum drifts with its length (16 x 128^2, 288 -> 160, 26,000
-    // pixels each: 1.8e-5 of the largest sum)
-    if (splitk < 1) gz = std::min<long long>(rows, std::max(gz, (npix + 8191) / 8192));
+    // and at most 4096 pixels in an accumulator: wide layers have many tiles and so few
+    // splits, and an FP32 sum drifts with its length (16 x 128^2: 1.8e-5 of the largest
+    // sum with 26,000 pixels each, over 1e-5 at 8192 still)
+    if (splitk < 1) gz = std::min<long long>(rows, std::max(gz, (npix + 4095) / 4096));
     if (gz > 65535) return false;
     CUtensorMap mx, my;
     {
