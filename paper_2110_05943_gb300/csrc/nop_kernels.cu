@@ -39,6 +39,14 @@ namespace {
 // in front of them has ended, and wait here before they touch its results.
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// What such a kernel reads may have been written while it was already running: coherent
+// loads behind the wait (not the read-only path, which wants the data unchanged for
+// the kernel's whole life; nor const __restrict__ parameters, which lead there).
+__device__ __forceinline__ uint4 ld_after_wait(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
 template <class... P, class... V>
 void launch_pdl(void (*k)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, const V&... v) {
     cudaLaunchConfig_t cfg = {};
@@ -618,7 +626,7 @@ __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sy
 // tile (output o = row * N + n0 + c0), bias from shared memory (sb: the
 // tile's first column), ReLU, mask, BF16 or FP32 store.
 __device__ __forceinline__ void tm_store8(const uint32_t* r, int o, int c0, int nt, const float* sb,
-                                          const __nv_bfloat16* __restrict__ mask, void* __restrict__ out,
+                                          const __nv_bfloat16* mask, void* __restrict__ out,
                                           int out_f32, int relu, int vec_out) {
     float v[8];
 #pragma unroll
@@ -663,9 +671,9 @@ __device__ __forceinline__ void tm_store8(const uint32_t* r, int o, int c0, int 
 // loads, the mask read before the accumulator is waited for (mk, 32 outputs
 // from c0 = 0) and applied to BF16 pairs.  FP32 sums and their rounding as in
 // tm_store8; about 150 instructions per 32 outputs against 600.
-__device__ __forceinline__ void tm_mask_load(const __nv_bfloat16* __restrict__ mask, int o, uint4 (&mk)[4]) {
+__device__ __forceinline__ void tm_mask_load(const __nv_bfloat16* mask, int o, uint4 (&mk)[4]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) mk[q] = __ldg(reinterpret_cast<const uint4*>(mask + o) + q);
+    for (int q = 0; q < 4; ++q) mk[q] = ld_after_wait(reinterpret_cast<const uint4*>(mask + o) + q);
 }
 // v where m > 0 (BF16 pairs; NaN counts as not greater), else 0
 __device__ __forceinline__ uint32_t tm_masked(uint32_t v, uint32_t m) {
@@ -673,7 +681,7 @@ __device__ __forceinline__ uint32_t tm_masked(uint32_t v, uint32_t m) {
     return v & __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&m), z);
 }
 __device__ __forceinline__ void tm_store_row32(uint32_t taddr, int o, int nt, const float* sb,
-                                               const __nv_bfloat16* __restrict__ mask, uint4 (&mk)[4],
+                                               const __nv_bfloat16* mask, uint4 (&mk)[4],
                                                __nv_bfloat16* __restrict__ out, int relu) {
     for (int c0 = 0; c0 < nt; c0 += 32) {
         uint32_t r[32];
@@ -717,7 +725,7 @@ __device__ __forceinline__ void tm_store_row32(uint32_t taddr, int o, int nt, co
 // Epilogue of one accumulator row (pixel `row`, outputs n0 .. n0 + nt - 1):
 // 32 columns per TMEM load and wait, then the rest 8 at a time.
 __device__ __forceinline__ void tm_store_row(uint32_t taddr, int row, int n0, int nt, int tile_n, int N,
-                                             const float* sb, const __nv_bfloat16* __restrict__ mask,
+                                             const float* sb, const __nv_bfloat16* mask,
                                              void* __restrict__ out, int out_f32, int relu, int vec_out) {
     const int o = row * N + n0;
     int c0 = 0;
@@ -743,8 +751,8 @@ __device__ __forceinline__ void tm_store_row(uint32_t taddr, int row, int n0, in
 template <int MODE, int kc>
 __global__ void __launch_bounds__(TM_THREADS, 2) k_conv_tma(const __grid_constant__ CUtensorMap mapA,
                                                          const __grid_constant__ CUtensorMap mapB,
-                                                         const float* __restrict__ bias,
-                                                         const __nv_bfloat16* __restrict__ mask, void* __restrict__ out,
+                                                         const float* bias,
+                                                         const __nv_bfloat16* mask, void* __restrict__ out,
                                                          int out_f32, int relu, ConvShape s, int M, int N, int tile_n,
                                                          int tmem_cols, int vec_out, int stages, int cchunks,
                                                          int ntiles, int ntn) {
@@ -918,7 +926,7 @@ __global__ void __launch_bounds__(TM_THREADS, 2) k_conv_tma(const __grid_constan
 template <int MODE, int NCH>
 __global__ void __launch_bounds__(TM_THREADS, 2)
     k_conv_row(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-               const float* __restrict__ bias, const __nv_bfloat16* __restrict__ mask, void* __restrict__ out, int out_f32,
+               const float* bias, const __nv_bfloat16* mask, void* __restrict__ out, int out_f32,
                int relu, ConvShape s, int N, int tile_n, int tmem_cols, int vec_out, int stages, int a_bytes, int total) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* const wsm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // weights, then the ring
@@ -2357,7 +2365,7 @@ __global__ void k_upcat8(const uint4* a, const uint4* b, uint4* __restrict__ y, 
 // holds the gradient of [up(a) | skip]; dx (n, h, w, ga) = sum of the four
 // copies of a's part, zeroed where a <= 0.  Rounded to BF16 before the mask as
 // the separate passes (split, upsampling backward, mask) did: the same bits.
-__global__ void k_up2_bwd_mask8(const uint4* dy, const uint4* __restrict__ a, uint4* __restrict__ dx, int n, int h, int w,
+__global__ void k_up2_bwd_mask8(const uint4* dy, const uint4* a, uint4* __restrict__ dx, int n, int h, int w,
                                 int ga, int gs) {
     pdl_start();
     pdl_wait();
@@ -2391,7 +2399,7 @@ __global__ void k_up2_bwd_mask8(const uint4* dy, const uint4* __restrict__ a, ui
 // (ds: gradient of [up | a], gs vectors per pixel, a's part from vector go):
 // dp / 4 (rounded to BF16, as the pooling's own backward pass gives it) + ds's
 // part, zeroed where a <= 0.
-__global__ void k_pool2_bwd_skip8(const uint4* dp, const uint4* ds, const uint4* __restrict__ a, uint4* __restrict__ dx, int n,
+__global__ void k_pool2_bwd_skip8(const uint4* dp, const uint4* ds, const uint4* a, uint4* __restrict__ dx, int n,
                                   int h, int w, int G, int gs, int go) {
     pdl_start();
     pdl_wait();
@@ -2537,9 +2545,9 @@ __global__ void __launch_bounds__(256) k_wgrad_small(const __nv_bfloat16* __rest
 // dx[p][ci] = sum_co dy[p][co] w[ci][co], zeroed where mask[p][ci] <= 0 (mask
 // may be NULL); one pixel per thread, the CIN x COUT weights in shared memory.
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) k_dgrad_small(const __nv_bfloat16* __restrict__ dy,
-                                                     const __nv_bfloat16* __restrict__ w,
-                                                     const __nv_bfloat16* __restrict__ mask,
+__global__ void __launch_bounds__(256) k_dgrad_small(const __nv_bfloat16* dy,
+                                                     const __nv_bfloat16* w,
+                                                     const __nv_bfloat16* mask,
                                                      __nv_bfloat16* __restrict__ dx, long long npix) {
     __shared__ float sw[CIN * COUT];
     pdl_start();
