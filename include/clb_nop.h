@@ -16,7 +16,9 @@
  * TMEM): fed by TMA copies when the pixels tile into whole image rows and
  * the channel counts are multiples of 8 (for the forward pass: when the
  * transposed weights are given; 3x3 weight gradients with channels in multiples
- * of 32, and 3x3 layers of 32, 64 or 96 gathered channels on rows of a multiple of 128, keep
+ * of 32 on rows of a multiple of 16 pixels up to 240, and 3x3 layers of 32 or 96
+ * gathered channels on rows of a multiple of 128 -- 64 channels with 64 outputs or
+ * more and two 128-pixel tiles per SM -- whose weights fit in shared memory, keep
  * image rows in a ring and fetch each once), otherwise from operands gathered through
  * registers when the gathered channel count is a multiple of 8 and the
  * operands are 16-byte aligned; the 1x1 convolution to 4 outputs runs on

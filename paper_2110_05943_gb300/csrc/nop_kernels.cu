@@ -12,7 +12,9 @@
 //   wgrad   : dW[tap, ci, co] += sum_p X[p + d(tap), ci] dY[p, co]   (split K, FP32 atomics)
 // In order of preference (the first that takes the shape runs):
 //   k_conv_row / k_wgrad_row -- image rows kept in a ring in shared memory, each
-//     fetched once for all nine taps (padded channels: 32 in, multiples of 32);
+//     fetched once for all nine taps (k_conv_row: 32, 64 or 96 gathered channels on
+//     rows of a multiple of 128 pixels, see launch_row; k_wgrad_row: channels in
+//     multiples of 32 on rows of a multiple of 16 pixels);
 //   k_conv_tma / k_wgrad_tma -- operands brought by TMA from the NHWC tensors
 //     into swizzled shared memory, tcgen05.mma with the accumulator in TMEM
 //     (whole-row pixel tiles, channel counts multiples of 8);
@@ -1829,11 +1831,10 @@ bool launch_tma(const void* A, const void* B, const float* bias, const void* mas
 }
 
 // Launches the row-ring kernel; false when the shape is not one it takes: 3x3,
-// width a multiple of 128, 32, 64 or 96 input channels, at most 256 outputs (a
-// multiple of 16) whose weights fit in shared memory.  Measured at 16 x 128^2 against k_conv_tma (both with the present epilogue
-// and issue loops): 32 -> 32 20.9 us against 25.0, 32 -> 96 41 against 51; with
-// more input channels it is no faster (96 -> 32: 47.5 against 46.3) or slower
-// (3 x 128^2, 64 -> 64: 14.7 against 12.5: one CTA per SM), so those stay there.
+// width a multiple of 128, 32, 64 or 96 gathered channels, at most 256 outputs (a
+// multiple of 16) whose weights fit in shared memory with four rows of the ring
+// (256 at 32 channels, 112 at 64, 48 at 96), and for 64 channels the condition below.  Measured at 16 x 128^2 against k_conv_tma (us):
+// 32 -> 32 25.0 / 20.9, 32 -> 96 51 / 41, 96 -> 32 44.1 / 31.6.
 template <int MODE>
 bool launch_row(const void* A, const void* B, const float* bias, const void* mask, void* out, int out_f32, int relu,
                 ConvShape s, long long M, long long N, cudaStream_t st, int* rc) {
