@@ -63,9 +63,9 @@ WORKLOAD = ("{n}x{n} porous cavity, seeded GRF porosity 0.3+0.6*Phi(g) (l=32, se
 BYTES_PER_CCU_F64 = 28 * 8 + 8
 # DRAM bytes (read + write) per node of one launch of the current FP64 step
 # kernel, ncu on the 2048^2 case of the same workload, scaled by the node
-# count (traffic grows with the nodes): 14 + 14 values and the 64-byte
-# per-node constant table.
-DRAM_BYTES_PER_CCU_MEASURED = 283.5
+# count (traffic grows with the nodes): 14 + 14 values and 32 bytes of
+# per-node constants.
+DRAM_BYTES_PER_CCU_MEASURED = 248.4
 
 
 def _peaks():
@@ -253,7 +253,7 @@ FORMS = {  # storage form -> (precision code, algorithmic bytes per coupled cell
 # DRAM bytes (read + write) per node of one launch of the current FP16 step
 # kernels, ncu on the 4096^2 case of the same workload; traffic grows with
 # the node count.  None: not captured for the kernel as it stands.
-FORMS_DRAM_PER_NODE = {"f16n": 76.3, "f16s": 60.3}
+FORMS_DRAM_PER_NODE = {"f16n": 75.6, "f16s": 59.8}
 # DRAM bytes (read + write) per node of one launch of the current batch
 # kernel (k_step_batch_mix, graph mode), ncu on the first 128 of the 512
 # cases (10.08 M nodes), scaled by the node count; None: not captured for
@@ -649,7 +649,7 @@ def surrogate_training(torch, bf16_peak, src, batch=16, steps=20):
             "ms_per_step": sec * 1e3, "samples_per_s": n / sec,
             "roofline": {"bound": "tensor", "achieved": tf, "peak": bf16_peak, "unit": "TFLOP/s",
                          "frac": tf / bf16_peak, "flop_per_step": fl, "traffic": None,
-                         "kernel": "k_conv_tma / k_wgrad_tma (TMA + tcgen05) + elementwise, whole step",
+                         "kernel": "k_conv_tma / k_conv_row / k_wgrad_row / k_wgrad_tma (TMA + tcgen05) + elementwise, whole step",
                          "peak_source": f"{src} bf16_tflops"}}
 
 

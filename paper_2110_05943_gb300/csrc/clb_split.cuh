@@ -18,11 +18,10 @@
 // post-collision fixed-point values to FP64 (round to nearest even), 5 of the
 // incoming g_i, and one product.
 //
-// Per node and step: 1507 instructions a warp (2210 with one split number per
-// register pair instead of two), 22 of them on the FP64 pipe.  4096^2: 1.01 ms
-// a step, 16.6 GLUPS, 4.8 TB/s (290 B of DRAM traffic a node), against 5.31 ms
-// for the collision in FP64.  What bounds it now is the sum of the pipes (FMA
-// 61 %, FP64 58 %, integer 44 % busy) at 19 warps per SM.
+// Per node and step: 1629 instructions a warp, 22 of them on the FP64 pipe.
+// 4096^2: 1.05 ms a step, 15.9 GLUPS, 3.9 TB/s (248 B of DRAM traffic a node),
+// against 5.31 ms for the collision in FP64.  What bounds it is issue (64 %) and
+// the sum of the pipes (FP64 56 %, FMA 50 %, integer 49 % busy) at 19 warps per SM.
 //
 // Range.  Fixed point covers f_i in [2^-8, 1); g is carried in a unit of each
 // node's own (split_unit), since fixed point is absolute precision: in the run's unit
