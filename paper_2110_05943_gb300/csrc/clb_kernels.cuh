@@ -1511,9 +1511,9 @@ __device__ __noinline__ void step_node_f64(const BufT<double>* in, const BufT<do
 // FP64 step launch shape: threads per block (x extent CLB_F64_BX) and the
 // resident blocks per SM the register allocation is capped for.  The FMA,
 // FP64-conversion and integer pipes are each about 60 % busy, so the step
-// wants warps to overlap them: 64 threads x 10 blocks (96 registers, 228
-// bytes of spills, 19 warps per SM) 1008 us at 4096^2, 128 x 5 1020, 128 x 4
-// (128 registers, no spills) 1062, 64 x 11 (80 registers) 1018.
+// wants warps to overlap them: 64 threads x 10 blocks (96 registers, spills in
+// the wall nodes' branch only, 19 warps per SM) 1031 us at 4096^2, 128 x 5 1035, 64 x 9
+// 1086, 64 x 11 (80 registers) 1093; with the constants from four planes 1055.
 #ifndef CLB_F64_THREADS
 #define CLB_F64_THREADS 64
 #endif
